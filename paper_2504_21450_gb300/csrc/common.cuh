@@ -232,35 +232,39 @@ __host__ __device__ inline WalkConst walk_const(double c)
 // where minxs = min_xorsign_abs.  When d0 and d1 differ in sign (a local extremum) u
 // and w are <= 0 and the cell sends g a, as CW84's flattening prescribes; otherwise
 // |u| = |minmod(d1, 2 d0)| and |w| = |minmod(d0, 2 d1)|.
+// d0 is held halved (h0), so that 2 d0 is 4 h0 and minxs(d0, 2 d1) is twice
+// minxs(h0, d1): scalings by powers of two, which are exact.
 template <bool kLimiter>
 struct Walk {
     float a1, a2;  // a_{p-1}, a_{p-2}
     float l1, l2;  // delta_{p-2}, delta_{p-3}
-    float d0;      // d0_{p-2}
+    float h0;      // d0_{p-2} / 2
     float o3;      // out_{p-3}
 
     __device__ __forceinline__ void reset()
     {
-        a1 = a2 = l1 = l2 = d0 = o3 = 0.0f;
+        a1 = a2 = l1 = l2 = h0 = o3 = 0.0f;
     }
 
     __device__ __forceinline__ float push(float a, const WalkConst& k)
     {
-        float dn = a - a1;                                          // delta_{p-1}
-        float e = fmaf(l2 - dn, 1.0f / 12.0f, 0.5f * l1);           // e_{p-2}
+        const float dn = a - a1;                                    // delta_{p-1}
+        const float h = 0.5f * l1;
+        const float e = fmaf(l2 - dn, 1.0f / 12.0f, h);             // e_{p-2}
+        const float B2 = k.B + k.B;
         float d1, out;
         if (kLimiter) {
             d1 = copysignf(fmaxf(min_xorsign_abs(e, l1), 0.0f), l1);
-            float u = min_xorsign_abs(d1, d0 + d0);
-            float w = min_xorsign_abs(d0, d1 + d1);
-            float xm = fmaxf(fmaf(k.A, u, k.B * w), 0.0f);
+            const float u = min_xorsign_abs(d1, 4.0f * h0);
+            const float w = min_xorsign_abs(h0, d1);                // half of minxs(d0, 2 d1)
+            const float xm = fmaxf(fmaf(k.A, u, B2 * w), 0.0f);
             out = fmaf(k.g, a2, copysignf(xm, d1));                 // out_{p-2}
         } else {
             d1 = e;
-            out = fmaf(k.B, d0, fmaf(k.A, d1, k.g * a2));
+            out = fmaf(B2, h0, fmaf(k.A, d1, k.g * a2));
         }
-        float res = (a2 - out) + o3;                                // new a_{p-2}
-        d0 = l1 - d1;                                               // d0_{p-1}
+        const float res = (a2 - out) + o3;                          // new a_{p-2}
+        h0 = fmaf(d1, -0.5f, h);                                    // d0_{p-1} / 2
         a2 = a1;
         a1 = a;
         l2 = l1;
@@ -284,47 +288,65 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 struct WalkConst2 {
-    float2 g, A, B;
+    float2 g, A, B2;  // B2 = 2 B
 };
 
 __device__ __forceinline__ WalkConst2 pack_const(const WalkConst& p, const WalkConst& q)
 {
-    return {make_float2(p.g, q.g), make_float2(p.A, q.A), make_float2(p.B, q.B)};
+    return {make_float2(p.g, q.g), make_float2(p.A, q.A), make_float2(p.B + p.B, q.B + q.B)};
+}
+// From two entries of a constant table (g, A, B, up).
+__device__ __forceinline__ WalkConst2 pack_const(const float4& p, const float4& q)
+{
+    return {make_float2(p.x, q.x), make_float2(p.y, q.y), make_float2(p.z + p.z, q.z + q.z)};
 }
 
-// Two Walks in lock step, lanes .x and .y; both must walk the same way.  Every
-// operation is the one Walk::push performs, in the same order, per lane.
-template <bool kLimiter>
+// Two Walks in lock step, lanes .x and .y; both must walk the same way.  The values are
+// those of Walk::push, bit for bit.
+// What bounds a push is operand reads: a packed instruction reads one 64-bit register
+// operand per cycle (measured: an fma with three distinct ones issues every 3.15 cycles, an
+// add every 2, a min or max every cycle), so of the packed forms only those that save
+// instructions by more than they cost are used, and the halved d0 takes one multiply out.
+// Cycles per push and scheduler with four warps (a loop of pushes): 37.6 before both
+// changes, 35.6 with them.  kForm: which of the two remaining fmas is written as two scalar
+// ones (0 none, 1 the limiter's, 2 the face value's); which is fastest depends on the
+// registers of the loop around it.  Plane-batched kernel: 1 (13.63 against 13.95 ms, 64x64x32
+// cells of the uniform workload); 3-pass kernel, 64x64x16 cells: 0 in FP32 (11.28 ms, form 1
+// 11.59, 2 11.34), 2 in bfloat16 (14.61 ms, form 0 14.80, 1 15.00).
+template <bool kLimiter, int kForm = 0>
 struct Walk2 {
-    float2 a1, a2, l1, l2, d0, o3;
+    float2 a1, a2, l1, l2, h0, o3;
 
     __device__ __forceinline__ void reset()
     {
-        a1 = a2 = l1 = l2 = d0 = o3 = make_float2(0.0f, 0.0f);
+        a1 = a2 = l1 = l2 = h0 = o3 = make_float2(0.0f, 0.0f);
     }
 
     __device__ __forceinline__ float2 push(float2 a, const WalkConst2& k)
     {
-        const float2 half = make_float2(0.5f, 0.5f), twelfth = make_float2(1.0f / 12.0f, 1.0f / 12.0f);
-        float2 dn = sub2(a, a1);
-        float2 e = fma2(sub2(l2, dn), twelfth, mul2(half, l1));
+        const float2 dn = sub2(a, a1);
+        const float2 h = mul2(l1, make_float2(0.5f, 0.5f));
+        const float2 t = sub2(l2, dn);
+        const float2 e = kForm == 2 ? make_float2(fmaf(t.x, 1.0f / 12.0f, h.x), fmaf(t.y, 1.0f / 12.0f, h.y))
+                                    : fma2(t, make_float2(1.0f / 12.0f, 1.0f / 12.0f), h);
         float2 d1, out;
         if (kLimiter) {
             d1.x = copysignf(fmaxf(min_xorsign_abs(e.x, l1.x), 0.0f), l1.x);
             d1.y = copysignf(fmaxf(min_xorsign_abs(e.y, l1.y), 0.0f), l1.y);
-            const float2 dd0 = add2(d0, d0), dd1 = add2(d1, d1);
+            const float2 dd0 = mul2(h0, make_float2(4.0f, 4.0f));
             const float2 u = make_float2(min_xorsign_abs(d1.x, dd0.x), min_xorsign_abs(d1.y, dd0.y));
-            const float2 w = make_float2(min_xorsign_abs(d0.x, dd1.x), min_xorsign_abs(d0.y, dd1.y));
-            float2 xm = fma2(k.A, u, mul2(k.B, w));
+            const float2 w = make_float2(min_xorsign_abs(h0.x, d1.x), min_xorsign_abs(h0.y, d1.y));
+            const float2 bw = mul2(k.B2, w);
+            float2 xm = kForm == 1 ? make_float2(fmaf(k.A.x, u.x, bw.x), fmaf(k.A.y, u.y, bw.y)) : fma2(k.A, u, bw);
             xm.x = copysignf(fmaxf(xm.x, 0.0f), d1.x);
             xm.y = copysignf(fmaxf(xm.y, 0.0f), d1.y);
             out = fma2(k.g, a2, xm);
         } else {
             d1 = e;
-            out = fma2(k.B, d0, fma2(k.A, d1, mul2(k.g, a2)));
+            out = fma2(k.B2, h0, fma2(k.A, d1, mul2(k.g, a2)));
         }
-        float2 res = add2(sub2(a2, out), o3);
-        d0 = sub2(l1, d1);
+        const float2 res = add2(sub2(a2, out), o3);
+        h0 = make_float2(fmaf(d1.x, -0.5f, h.x), fmaf(d1.y, -0.5f, h.y));
         a2 = a1;
         a1 = a;
         l2 = l1;

@@ -582,16 +582,10 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
         const bool zv0 = zcx < it.ex && zcr < it.er, zv1 = zcx < it.ex && zcr + 8 < it.er;
         const int zoff = (kHalo + zcr) * kRP + (kHalo + zcx) * kChunk + 4 * zq;
         const int64_t zcell = (int64_t)(it.tx0 + zcx) + (int64_t)(it.tr0 + zcr) * str_r;  // at plane 0
-        Walk2<kLim> zw[4];
+        Walk2<kLim, 1> zw[4];
 #pragma unroll
         for (int i = 0; i < 4; i++) zw[i].reset();
-        WalkConst2 kz;
-        {
-            const float4 c = S.kc[2][4 * zq];  // the streamed axis is not x: equal over vx
-            kz.g = make_float2(c.x, c.x);
-            kz.A = make_float2(c.y, c.y);
-            kz.B = make_float2(c.z, c.z);
-        }
+        const WalkConst2 kz = pack_const(S.kc[2][4 * zq], S.kc[2][4 * zq]);  // the streamed axis is not x: equal over vx
 
         if (stager && !pref) stage_batch<kCodec, kA0X>(P, S, it, ti, 0, gb, sl);
         int k = 0;
@@ -610,8 +604,7 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
                 const int j = tid / (kLines * 8), rem = tid - j * (kLines * 8);
                 const int line = rem >> 3, l0 = 2 * (rem & 7);
                 if (j < nj) {
-                    const float4 c0 = S.kc[0][l0], c1 = S.kc[0][l0 + 1];
-                    const WalkConst2 kx{make_float2(c0.x, c1.x), make_float2(c0.y, c1.y), make_float2(c0.z, c1.z)};
+                    const WalkConst2 kx = pack_const(S.kc[0][l0], S.kc[0][l0 + 1]);
                     float* p = B + j * kPS + (line + (up1 ? 0 : 1)) * kS1 + l0;
                     // 16-bit storage: chunk scales of the line's cells
                     const float* ps = scales_of(S) + (slot * kNB + j) * kE * kSP + (line + (up1 ? 0 : 1)) * kC1;
@@ -631,7 +624,7 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
                             return dec2<kCodec>(w, make_float2(sc, sc));
                         }
                     };
-                    Walk2<kLim> wk;
+                    Walk2<kLim, 1> wk;
                     wk.reset();
                     if (up0) {
 #pragma unroll
@@ -669,10 +662,9 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
                 const int j = tid >> 7, rem = tid & 127;
                 const int line = rem >> 3, l0 = 2 * (rem & 7);
                 if (j < nj) {
-                    const float4 c0 = S.kc[1][l0], c1 = S.kc[1][l0 + 1];
-                    const WalkConst2 ky{make_float2(c0.x, c1.x), make_float2(c0.y, c1.y), make_float2(c0.z, c1.z)};
+                    const WalkConst2 ky = pack_const(S.kc[1][l0], S.kc[1][l0 + 1]);
                     float* p = B + j * kPS + (kHalo + line) * kS0 + l0;
-                    Walk2<kLim> wk;
+                    Walk2<kLim, 1> wk;
                     wk.reset();
                     if (up1) {
 #pragma unroll
