@@ -791,12 +791,13 @@ void launch_items_from_flags(Grid* g, int64_t ntiles, bool flat)
 }
 
 // Work list of a fused launch: one item per (block id, tile column) holding any slot of
-// the next layout, grouped by block id (item_base[b] .. item_base[b+1]).
-void launch_tile_list(Grid* g, const TileArgs& T, int64_t need, int64_t ntiles)
+// the next layout, grouped by block id (item_base[b] .. item_base[b+1]); flat as in
+// launch_items_from_flags.
+void launch_tile_list(Grid* g, const TileArgs& T, int64_t need, int64_t ntiles, bool flat)
 {
     k_tile_flags<<<nblk(need, 256), 256, 0, g->stream>>>(T, g->tile_flags);
     note_launch();
-    launch_items_from_flags(g, ntiles, false);
+    launch_items_from_flags(g, ntiles, flat);
 }
 
 // Work-list buffers for `need` (block id, tile) pairs (allocated before any captured
@@ -856,7 +857,7 @@ vl_status run_fused(Grid* g, const StepArgs& a)
     T.ntile0 = ntile0;
     T.ntile1 = ntile1;
     T.ty = ty;
-    launch_tile_list(g, T, need, ntiles);
+    launch_tile_list(g, T, need, ntiles, false);
 
     FusedArgs P;
     P.G = G;

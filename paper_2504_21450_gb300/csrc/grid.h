@@ -198,7 +198,7 @@ struct TileArgs {
     int ntile0, ntile1;
     int ty;
 };
-void launch_tile_list(Grid* g, const TileArgs& T, int64_t need, int64_t ntiles);
+void launch_tile_list(Grid* g, const TileArgs& T, int64_t need, int64_t ntiles, bool flat);
 // gt3.cu: the plane-batched GT3 kernel (GT3, streamed axis y or z, no
 // velocity block straddling v_d = 0)
 bool gt3_applies(const Grid* g, const StepArgs& a);

@@ -6,15 +6,20 @@
 // staged into shared memory plane by plane along the third (streamed) axis, exactly once
 // per step, and all three sweeps run on it.  What differs is how the work is laid out on
 // the SM:
-//   * planes are processed in batches of three.  While the CTA sweeps batch k, the four
-//     warps that sit out sweep 1 stage batch k+1, one halo row per thread, with TMA bulk
-//     copies (one per contiguous run of a row; 16-byte cp.async for the short run where a
-//     dense row wraps around the periodic grid).  The CTA synchronises once per batch
-//     after sweep 0; after sweep 1 the sweep-1 warps only arrive on a named barrier that
-//     the staging warps wait on, and go on to sweep 2 among themselves;
+//   * planes are processed in batches of three, in two batch buffers.  Sixteen warps sweep;
+//     four more stage, up to two batches ahead and across items, with TMA bulk copies (one
+//     per contiguous run of a row; 16-byte cp.async for the short run where a dense row
+//     wraps around the periodic grid).  A batch's mbarrier tells the sweeping warps that it
+//     is staged, a second one tells the staging warps that it is swept.  (Until the staging
+//     had warps of its own, the four warps that sit out sweep 1 did it; on sparse and 16-bit
+//     states it took 7000-8400 cycles of a 13000-cycle batch and the others waited: 19.5
+//     against 16.2 ms per step on 128x32x16 cells of the shock, 10.3 against 8.8 ms in
+//     bfloat16 on 64x64x16 cells of the uniform workload; dense FP32 is as fast either way.)
+//     The sweeping warps synchronise twice a batch, after sweep 0 and after sweep 1;
 //   * every walk moves two velocity cells in packed f32x2 registers: sweep 0 runs on the
 //     21 halo lines that sweep 1 reads (3 planes x 21 lines x 8 lane pairs = 504 walks),
-//     sweep 1 on the 16 tile lines (384 walks), both in place in shared memory;
+//     sweep 1 on the 16 tile lines (384 walks), both in place in shared memory.  Only the
+//     21 x 21 cells that the walks read are staged;
 //   * sweep 2 is streamed: each compute thread keeps the windows of four velocity cells
 //     (one vx row of a chunk) of two tile cells in registers, reads them with 16-byte
 //     shared loads and writes 16-byte global stores, so a warp writes 8 whole cells.
@@ -35,37 +40,56 @@ namespace {
 
 constexpr int kT = 16;                      // tile edge along both in-plane axes
 constexpr int kE = kT + 2 * kHalo;          // 22 staged cells per in-plane axis
+constexpr int kNB = 3;                      // planes per batch
+constexpr int kNC = 512;                    // sweeping threads (warps 0-15)
+constexpr int kNS = 128;                    // staging threads (warps 16-19)
+constexpr int kNT = kNC + kNS;
+// Registers per thread: the CTA is launched with 96 (640 threads); the staging warps give
+// some back and the sweeping ones take them: 512 x 104 + 128 x 64 = 640 x 96.  (112 and 32
+// make the staging code spill; 13.94 against 13.98 ms on 64x64x32 cells.)
+constexpr int kRegsSweep = 104, kRegsStage = 64;
+static_assert(kNC * kRegsSweep + kNS * kRegsStage <= kNT * 96, "register split within the launch's total");
+constexpr int kLines = kT + 5;              // sweep-0 lines: those sweep 1 reads
+constexpr int kFirst = kHalo + 2;           // first streamed plane that completes an output
+
 constexpr int kRP = kE * kChunk + 16;       // staged row pitch in floats: rows 16 banks apart
 constexpr int kPS = kE * kRP + 16;          // plane pitch in floats
-constexpr int kNB = 3;                      // planes per batch
-constexpr int kNC = 512;                    // threads (16 warps)
-constexpr int kNT = kNC;
-constexpr int kLines = kT + 5;              // sweep-0 lines: those sweep 1 reads
 constexpr int kNX = kNB * kLines * 8;       // sweep-0 walks per batch (lane pairs)
 constexpr int kNY = kNB * kT * 8;           // sweep-1 walks per batch
-constexpr int kNS = kNC - kNY;              // staging threads: those that sit out sweep 1
-constexpr int kFirst = kHalo + 2;           // first streamed plane that completes an output
+static_assert(kNX <= kNC && kNY <= kNC, "walks of a batch must fit the threads");
+static_assert(kT * kT * 4 == 2 * kNC, "sweep 2: two tile cells x one vx row per thread");
 // 16-bit storage with sweep 0 along x: the codes of a staged row are packed (8 floats per
 // cell) at the end of the row that sweep 0 reaches last -- from float kCodesHi when it
 // walks up, from float 0 when it walks down
 constexpr int kCodesHi = kRP - kE * kChunk / 2;
-static_assert(kNX <= kNC && kNY <= kNC, "walks of a batch must fit the compute threads");
-static_assert(kT * kT * 4 == 2 * kNC, "sweep 2: two tile cells x one vx row per thread");
-static_assert(kNS == 128, "staging threads: warps 12-15 (named barrier 1)");
+
+// One work item: block id b, velocity chunk q, tile origin and extent.
+struct Item {
+    int b, q, tx0, tr0, ex, er;
+    int dense_in, dense_out, up0, up1, up2;
+    int64_t ibase, obase, okeep;
+};
+
+// What the threads read for an item: its staged rows and its sweep constants.
+struct ItemTables {
+    float4 kc[3][kChunk];  // WalkConst (g, A, B, up) per sweep and velocity cell
+    int run[kE][3];        // contiguous runs of a staged row along x: first column, x, length
+    int rrow[kE];          // row-space part of each row
+    int xs[kE];            // x of each column
+    int nrun;
+    int r0, u0;            // first staged row and column (kLines of each are staged)
+};
 
 struct Gt3Smem {
     float buf[2][kNB][kPS];   // staged planes, swept in place (two batches in flight)
     int orank[2][kNB][kT * kT];  // sparse output slots of the tile cells, per plane
-    float4 kc[3][kChunk];     // WalkConst (g, A, B, up) per sweep and velocity cell
-    int run[2][kE][3];        // per item parity: contiguous runs of a staged row along x
-    int rrow[2][kE];          // per item parity: row-space part of each staged row
-    int xs[2][kE];            // per item parity: x of each staged column
-    uint64_t bar[2];          // staging barriers, one per batch buffer
-    long long work;           // the current work item
-    long long next;           // the one after it (taken while the current one runs)
-    int nrun[2];
-    int pref;                 // batch 0 of the current item was staged during the last one
-    int abort;
+    Item item[2];             // per item parity, like the tables and the work index
+    ItemTables tab[2];
+    long long work[2];
+    uint64_t bar[2];          // per batch buffer: staged
+    uint64_t empty[2];        // per batch buffer: swept, may be staged again
+    int abort;                // a sweeping warp's wait ran out
+    int late;                 // the staging warps' wait ran out
 };
 // 16-bit storage: the chunk scales of the staged cells, [2][kNB][kE][kSP] floats after
 // Gt3Smem (per batch buffer and plane, staged row-major like the cells).  The row pitch
@@ -87,8 +111,9 @@ struct Gt3Args {
     int nvmax;
     float thr;
     int ntile0;         // tiles along x
-    const uint32_t* items;
-    const int64_t* item_base;  // [nb + 1]
+    uint32_t ntiles;    // tiles per block id
+    const uint32_t* items;   // (block id, tile) pairs as b * ntiles + tile, in that order
+    const int64_t* npairs;   // their number
     uint8_t* keepq;
     StepCounters* ctr;
     int report_late;    // testing hook: a staging wait not complete at its first poll is
@@ -197,6 +222,7 @@ constexpr uint64_t kWaitLimitNs = 1000000000ull;
 
 __device__ __forceinline__ bool bar_wait_bounded(uint64_t* bar, unsigned parity)
 {
+    if (bar_try(bar, parity)) return true;
     unsigned polls = 0;
     const uint64_t t0 = now_ns();
     while (!bar_try(bar, parity)) {
@@ -211,69 +237,82 @@ __device__ __forceinline__ void sts2(float* p, float2 v) { *reinterpret_cast<flo
 // row-space contribution (row = y + ny*z) of coordinate c along physical axis d (1 or 2)
 __device__ __forceinline__ int rowpart(int d, int c, int ny) { return d == 1 ? c : c * ny; }
 
-// One work item: block id b, velocity chunk q, tile origin and extent.
-struct Item {
-    int b, q, tx0, tr0, ex, er;
-    bool dense_in, dense_out, up0, up2;
-    int64_t ibase, obase;
-};
-
-__device__ __forceinline__ Item decode_item(const Gt3Args& P, int64_t w)
+// Named barriers: the staging warps, the sweeping warps.
+constexpr int kBarStage = 1, kBarSweep = 2;
+__device__ __forceinline__ void named_sync(int id, int n)
+{
+    asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory");
+}
+// Item w of the list: chunk w % 4 of pair w / 4.
+__device__ __forceinline__ void decode_item(const Gt3Args& P, int64_t w, Item& it)
 {
     const GridGeom& G = P.G;
-    int lo = 0, hb = G.nb;  // items are grouped by b, q-major then tile
-    while (hb - lo > 1) {
-        const int mid = (lo + hb) >> 1;
-        if (4 * P.item_base[mid] <= w) lo = mid;
-        else hb = mid;
-    }
-    Item it;
-    it.b = lo;
-    const int64_t mb = P.item_base[lo + 1] - P.item_base[lo];
-    const int64_t wl = w - 4 * P.item_base[lo];
-    it.q = (int)(wl / mb);
-    const uint32_t tile = P.items[P.item_base[lo] + (wl % mb)];
+    const uint32_t pair = P.items[w >> 2];
+    const int b = (int)(pair / P.ntiles);
+    const uint32_t tile = pair - (uint32_t)b * P.ntiles;
+    const int q = (int)(w & 3);
+    it.b = b;
+    it.q = q;
     it.tx0 = (int)(tile % P.ntile0) * kT;
     it.tr0 = (int)(tile / P.ntile0) * kT;
     it.ex = min(kT, G.n[0] - it.tx0);
     it.er = min(kT, G.n[P.ar] - it.tr0);
-    it.dense_in = (P.in.dense[lo] & 3) == 3;
-    it.dense_out = (P.out.dense[lo] & 1) != 0;
-    it.ibase = ((int64_t)P.in.base[lo] * 4 + (int64_t)it.q * P.in.cnt[lo]) * kChunk;
-    it.obase = ((int64_t)P.out.base[lo] * 4 + (int64_t)it.q * P.out.cnt[lo]) * kChunk;
-    // direction along the streamed axis (not x: the same for every velocity cell of the
-    // item, the host checks that no block straddles v = 0)
-    const int d = P.ax[2];
-    const int bc = d == 1 ? (lo / G.nbx) % G.nby : lo / (G.nbx * G.nby);
-    it.up2 = P.walk[d * P.nvmax + bc * 4 + (d == 2 ? it.q : 0)].w != 0.0f;
-    // and along the axis of sweep 0 (uniform for the same reason)
-    const int d0 = P.ax[0];
-    const int bc0 = d0 == 0 ? lo % G.nbx : (d0 == 1 ? (lo / G.nbx) % G.nby : lo / (G.nbx * G.nby));
-    it.up0 = P.walk[d0 * P.nvmax + bc0 * 4 + (d0 == 2 ? it.q : 0)].w != 0.0f;
-    return it;
+    it.dense_in = (P.in.dense[b] & 3) == 3;
+    it.dense_out = (P.out.dense[b] & 1) != 0;
+    it.ibase = ((int64_t)P.in.base[b] * 4 + (int64_t)q * P.in.cnt[b]) * kChunk;
+    it.okeep = (int64_t)P.out.base[b];
+    it.obase = (it.okeep * 4 + (int64_t)q * P.out.cnt[b]) * kChunk;
+    // directions along the three sweep axes: the same for every velocity cell of the item
+    // (the host checks that no block straddles v = 0)
+    const int bc[3] = {b % G.nbx, (b / G.nbx) % G.nby, b / (G.nbx * G.nby)};
+    int up[3];
+    for (int j = 0; j < 3; j++) {
+        const int d = P.ax[j];
+        up[j] = P.walk[d * P.nvmax + bc[d] * 4 + (d == 2 ? q : 0)].w != 0.0f;
+    }
+    it.up0 = up[0];
+    it.up1 = up[1];
+    it.up2 = up[2];
 }
 
-// Runs and row parts of an item's staged rows and the x of its staged columns into
-// table t (threads kNC-1-2kE .. kNC-1).
-__device__ __forceinline__ void item_tables(const Gt3Args& P, Gt3Smem& S, const Item& it, int t, int tid)
+// The tables of an item (the staging threads, sl = 0 .. kNS-1).
+__device__ __forceinline__ void item_tables(const Gt3Args& P, const Item& it, ItemTables& t, int sl)
 {
-    const int nx = P.G.n[0], nr = P.G.n[P.ar];
-    if (tid >= kNC - 1 - 2 * kE && tid < kNC - 1 - kE) S.xs[t][tid - (kNC - 1 - 2 * kE)] = wrapi(it.tx0 - kHalo + tid - (kNC - 1 - 2 * kE), nx);
-    if (tid == kNC - 1) {
-        int u0 = 0, nrun = 0;
-        while (u0 < kE) {
-            const int x = wrapi(it.tx0 - kHalo + u0, nx);
-            const int len = min(kE - u0, nx - x);
-            S.run[t][nrun][0] = u0;
-            S.run[t][nrun][1] = x;
-            S.run[t][nrun][2] = len;
-            nrun++;
-            u0 += len;
+    const GridGeom& G = P.G;
+    const int nx = G.n[0], nr = G.n[P.ar];
+    for (int i = sl; i < 3 * kChunk + 2 * kE + 1; i += kNS) {
+        if (i < 3 * kChunk) {
+            // sweep constants of the item's 16 velocity cells (v = vx + 4 vy, vz = q)
+            const int j = i >> 4, l = i & 15;
+            const int d = P.ax[j];
+            const int bc = d == 0 ? it.b % G.nbx : (d == 1 ? (it.b / G.nbx) % G.nby : it.b / (G.nbx * G.nby));
+            const int wi = d == 0 ? (l & 3) : (d == 1 ? (l >> 2) : it.q);
+            t.kc[j][l] = P.walk[d * P.nvmax + bc * 4 + wi];
+        } else if (i < 3 * kChunk + kE) {
+            const int u = i - 3 * kChunk;
+            t.xs[u] = wrapi(it.tx0 - kHalo + u, nx);
+        } else if (i < 3 * kChunk + 2 * kE) {
+            const int u = i - 3 * kChunk - kE;
+            t.rrow[u] = rowpart(P.ar, wrapi(it.tr0 - kHalo + u, nr), G.n[1]);
+        } else {
+            // a walk reads 3 cells upwind of the tile and 2 downwind of it, so one of the
+            // outermost rows and columns is not needed
+            const bool x_first = P.ax[0] == 0;
+            t.r0 = (x_first ? it.up1 : it.up0) ? 0 : 1;
+            t.u0 = (x_first ? it.up0 : it.up1) ? 0 : 1;
+            int u0 = t.u0, nrun = 0;
+            const int end = u0 + kLines;
+            while (u0 < end) {
+                const int x = wrapi(it.tx0 - kHalo + u0, nx);
+                const int len = min(end - u0, nx - x);
+                t.run[nrun][0] = u0;
+                t.run[nrun][1] = x;
+                t.run[nrun][2] = len;
+                nrun++;
+                u0 += len;
+            }
+            t.nrun = nrun;
         }
-        S.nrun[t] = nrun;
-    } else if (tid >= kNC - 1 - kE && tid < kNC - 1) {
-        const int u = tid - (kNC - 1 - kE);
-        S.rrow[t][u] = rowpart(P.ar, wrapi(it.tr0 - kHalo + u, nr), P.G.n[1]);
     }
 }
 
@@ -293,17 +332,17 @@ __device__ __forceinline__ void item_tables(const Gt3Args& P, Gt3Smem& S, const 
 constexpr int kShortRun = 4;
 
 // cells of an item's staged row that go by bulk copies (runs longer than kShortRun)
-__device__ __forceinline__ int bulk_cells(const Gt3Smem& S, int t)
+__device__ __forceinline__ int bulk_cells(const ItemTables& t)
 {
     int c = 0;
-    for (int k2 = 0; k2 < S.nrun[t]; k2++)
-        if (S.run[t][k2][2] > kShortRun) c += S.run[t][k2][2];
+    for (int k2 = 0; k2 < t.nrun; k2++)
+        if (t.run[k2][2] > kShortRun) c += t.run[k2][2];
     return c;
 }
 
 template <int kCodec, bool kA0X>
-__device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const Item& it, int t, int k,
-                                            unsigned g, int sl)
+__device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const Item& it,
+                                            const ItemTables& t, int k, unsigned g, int sl)
 {
     const GridGeom& G = P.G;
     const int nx = G.n[0], ny = G.n[1], a2 = P.ax[2], n2 = G.n[a2];
@@ -311,7 +350,7 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
     const unsigned slot = g & 1u;
     uint64_t* bar = &S.bar[slot];
     const int nj = min(kNB, nsteps - kNB * k);
-    const int nrun = S.nrun[t];
+    const int nrun = t.nrun;
     // staged row (and output row) of this thread: rows go round-robin over the four
     // staging warps, whose lanes issue their copies one after another
     const int sw = (sl & 31) * (kNS / 32) + (sl >> 5);
@@ -322,10 +361,10 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
         using T = typename Codec<kCodec>::T;
         const T* cpool = static_cast<const T*>(P.in.pool) + it.ibase;  // codes of rank 0
         const float* spool = P.in.scale + it.ibase / kChunk;            // scale of rank 0
-        if (sw < nj * kE) {
-            const int j = sw / kE, rho = sw - j * kE;
+        if (sw < nj * kLines) {
+            const int j = sw / kLines, rho = t.r0 + sw - j * kLines;
             const int pz = wrapi(plane_of(kNB * k + j), n2);
-            const int64_t row = (int64_t)S.rrow[t][rho] + rowpart(a2, pz, ny);
+            const int64_t row = (int64_t)t.rrow[rho] + rowpart(a2, pz, ny);
             float* drow = &S.buf[slot][j][rho * kRP];
             float* srow = scales_of(S) + ((slot * kNB + j) * kE + rho) * kSP;
             if constexpr (kA0X) {
@@ -334,7 +373,7 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
                 if (it.dense_in) {
                     const int64_t r0 = row * nx;
                     for (int k2 = 0; k2 < nrun; k2++) {
-                        const int u0 = S.run[t][k2][0], x0 = S.run[t][k2][1], len = S.run[t][k2][2];
+                        const int u0 = t.run[k2][0], x0 = t.run[k2][1], len = t.run[k2][2];
                         float* d = codes + u0 * (kChunk / 2);
                         const T* src = cpool + (r0 + x0) * kChunk;
                         if (len > kShortRun) {
@@ -343,13 +382,13 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
                             for (int i = 0; i < len * 2; i++) cp16(d + 4 * i, src + 8 * i, 16);
                         }
                     }
-                    for (int u = 0; u < kE; u++) cp4(srow + u, spool + r0 + S.xs[t][u], 4);
+                    for (int u = t.u0; u < t.u0 + kLines; u++) cp4(srow + u, spool + r0 + t.xs[u], 4);
                 } else {
                     // runs of present cells (consecutive slots) as bulk copies, each announced
                     // to the barrier before it is issued; absent cells get zero codes and scale
                     const int64_t wbase = (int64_t)it.b * G.RW + row * G.W;
                     for (int k2 = 0; k2 < nrun; k2++) {
-                        const int u0 = S.run[t][k2][0], x0 = S.run[t][k2][1], len = S.run[t][k2][2];
+                        const int u0 = t.run[k2][0], x0 = t.run[k2][1], len = t.run[k2][2];
                         const int w0 = x0 >> 6, sh = x0 & 63;
                         const bool two = sh + len > 64;
                         const uint64_t ua = P.in.ubits[wbase + w0];
@@ -384,8 +423,8 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
                     }
                 }
             } else {
-                for (int u = 0; u < kE; u++) {
-                    const int x = S.xs[t][u];
+                for (int u = t.u0; u < t.u0 + kLines; u++) {
+                    const int x = t.xs[u];
                     int64_t r;
                     if (it.dense_in) {
                         r = row * nx + x;
@@ -408,22 +447,22 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
         // dense rows with sweep 0 along x: the batch's code bytes, announced without an
         // arrival (the phase also waits for every staging thread's arrival below)
         if (kA0X && it.dense_in && sl == 0)
-            bar_add_tx(bar, (unsigned)(nj * kE * bulk_cells(S, t) * kChunk * sizeof(T)));
+            bar_add_tx(bar, (unsigned)(nj * kLines * bulk_cells(t) * kChunk * sizeof(T)));
         cp_arrive(bar);
     } else if (it.dense_in) {
         // the batch's bulk-copy bytes, announced once (the copies of the other staging
         // threads may complete before or after it; the phase also waits for every staging
         // thread's arrival)
-        if (sl == 0) bar_add_tx(bar, (unsigned)(nj * kE * bulk_cells(S, t) * kChunk * sizeof(float)));
-        if (sw < nj * kE) {
-            const int j = sw / kE, rho = sw - j * kE;
+        if (sl == 0) bar_add_tx(bar, (unsigned)(nj * kLines * bulk_cells(t) * kChunk * sizeof(float)));
+        if (sw < nj * kLines) {
+            const int j = sw / kLines, rho = t.r0 + sw - j * kLines;
             const int pz = wrapi(plane_of(kNB * k + j), n2);
-            const int64_t row = (int64_t)S.rrow[t][rho] + rowpart(a2, pz, ny);
+            const int64_t row = (int64_t)t.rrow[rho] + rowpart(a2, pz, ny);
             const float* src = ipool + it.ibase + row * nx * kChunk;
             float* dst = &S.buf[slot][j][rho * kRP];
             fence_async_smem();
             for (int k2 = 0; k2 < nrun; k2++) {
-                const int u0 = S.run[t][k2][0], x0 = S.run[t][k2][1], len = S.run[t][k2][2];
+                const int u0 = t.run[k2][0], x0 = t.run[k2][1], len = t.run[k2][2];
                 if (len > kShortRun) {
                     copy_g2s(dst + u0 * kChunk, src + x0 * kChunk, (unsigned)(len * kChunk * sizeof(float)), bar);
                 } else {
@@ -438,15 +477,15 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
         // barrier before it is issued; absent cells are zeroed.  Each staging thread
         // arrives after announcing its bytes, so the phase cannot end before every
         // announcement.
-        if (sw < nj * kE) {
-            const int j = sw / kE, rho = sw - j * kE;
+        if (sw < nj * kLines) {
+            const int j = sw / kLines, rho = t.r0 + sw - j * kLines;
             const int pz = wrapi(plane_of(kNB * k + j), n2);
-            const int64_t row = (int64_t)S.rrow[t][rho] + rowpart(a2, pz, ny);
+            const int64_t row = (int64_t)t.rrow[rho] + rowpart(a2, pz, ny);
             const int64_t wbase = (int64_t)it.b * G.RW + row * G.W;
             float* dst = &S.buf[slot][j][rho * kRP];
             fence_async_smem();
             for (int k2 = 0; k2 < nrun; k2++) {
-                const int u0 = S.run[t][k2][0], x0 = S.run[t][k2][1], len = S.run[t][k2][2];
+                const int u0 = t.run[k2][0], x0 = t.run[k2][1], len = t.run[k2][2];
                 const int w0 = x0 >> 6, sh = x0 & 63;
                 const bool two = sh + len > 64;
                 const uint64_t ua = P.in.ubits[wbase + w0];
@@ -484,9 +523,9 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
         }
         bar_arrive(bar);
     }
-    // output slots of the tile cells of a sparse next layout
-    if (!it.dense_out && sw < nj * kT) {
-        const int j = sw / kT, rr = sw - j * kT;
+    // output slots of the tile cells of a sparse next layout, two threads per tile row
+    if (!it.dense_out && sw < nj * 2 * kT) {
+        const int j = sw / (2 * kT), rr = (sw >> 1) - j * kT;
         const int s = kNB * k + j;
         if (s >= kFirst) {
             const int zo = out_of(s);
@@ -500,13 +539,65 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
                 ow = P.out.woff[wi];
             }
 #pragma unroll
-            for (int i = 0; i < kT; i++) {
+            for (int i8 = 0; i8 < kT / 2; i8++) {
+                const int i = (sw & 1) * (kT / 2) + i8;
                 const int bit = (it.tx0 + i) & 63;  // the 16 cells share one bitmap word
                 const bool has = i < it.ex && ((uw >> bit) & 1ull);
                 orow[i] = has ? (int)(ow + __popcll(uw & ((1ull << bit) - 1ull))) : -1;
             }
         }
     }
+}
+
+// The staging warps: they run up to two batches ahead of the sweeping warps, across
+// items.  The index of the next item is taken one item ahead.
+template <bool kA0X, int kCodec>
+__device__ __forceinline__ void stage_loop(const Gt3Args& P, Gt3Smem& S, int sl, int nbatch, int64_t nwork)
+{
+    long long wnext = 0;
+    if (sl == 0) wnext = (long long)atomicAdd(&P.ctr->work_next, 1ull);
+    // Buffer g & 1 is free once batch g - 2 is swept; the sweeping warps have then also left
+    // the item before the one of that batch, whose description and tables are overwritten.
+    // One thread waits, and the others learn of it at the staging warps' barrier.
+    auto wait_empty = [&](unsigned g) {
+        if (g >= 2 && sl == 0 && !bar_wait_bounded(&S.empty[g & 1u], ((g >> 1) - 1u) & 1u)) S.late = 1;
+    };
+    unsigned g = 0;
+    bool late = false;
+    for (int par = 0; !late; par ^= 1) {
+        wait_empty(g);
+        if (sl == 0) {
+            S.work[par] = wnext;
+            if (wnext < nwork && !S.late) {
+                decode_item(P, wnext, S.item[par]);
+                wnext = (long long)atomicAdd(&P.ctr->work_next, 1ull);
+            }
+        }
+        named_sync(kBarStage, kNS);
+        late = S.late != 0;
+        if (late) break;
+        if (S.work[par] >= nwork) {
+            // nothing more to stage: the phase completes and tells the sweeping warps to end
+            bar_arrive(&S.bar[g & 1u]);
+            if (sl == 0) bar_arrive(&S.bar[g & 1u]);
+            return;
+        }
+        const Item& it = S.item[par];
+        item_tables(P, it, S.tab[par], sl);
+        for (int k = 0; k < nbatch; k++, g++) {
+            if (k > 0) wait_empty(g);
+            named_sync(kBarStage, kNS);
+            late = S.late != 0;
+            if (late) break;
+            // the plain arrival publishes the item's description and tables; the others
+            // may be deferred until a thread's copies land
+            if (sl == 0) bar_arrive(&S.bar[g & 1u]);
+            stage_batch<kCodec, kA0X>(P, S, it, S.tab[par], k, g, sl);
+        }
+    }
+    // the sweeping warps stopped: leave no copy in flight (the last two batches staged)
+    if (sl == 0) atomicOr(&P.ctr->error, 4);
+    for (unsigned i = 1; i <= 2 && i <= g; i++) bar_wait_bounded(&S.bar[(g - i) & 1u], ((g - i) >> 1) & 1u);
 }
 
 template <bool kLim, bool kA0X, int kCodec>
@@ -518,14 +609,13 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
     if (aborted(G.abort)) return;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
-    const bool stager = tid >= kNY;   // warps 12-15: stage the next batch during sweep 1
-    const int sl = tid - kNY;         // staging lane 0..127
     const int ar = P.ar, a2 = P.ax[2];
     const int n2 = G.n[a2];
     const int nsteps = n2 + kFirst;       // planes streamed per item (3 before, 2 after)
-    const int nbatch = (nsteps + kNB - 1) / kNB;
-    const int64_t nwork = 4 * P.item_base[G.nb];
-    const int64_t str_r = P.stride[ar], str_2 = P.stride[a2];
+    const int nbatch = (nsteps + kNB - 1) / kNB;  // at least 2
+    const int64_t nwork = 4 * *P.npairs;
+    const int str_r = (int)P.stride[ar], str_2 = (int)P.stride[a2];
+    const unsigned zrow8 = 8u * (unsigned)str_r;
     // staged offsets of a position along sweep axis 0 / 1 (in floats)
     constexpr int kS0 = kA0X ? kChunk : kRP;
     constexpr int kS1 = kA0X ? kRP : kChunk;
@@ -534,69 +624,68 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
     constexpr int kC1 = kA0X ? kSP : 1;
 
     if (tid == 0) {
-        // one arrival per staging thread
-        bar_init(&S.bar[0], kNS);
-        bar_init(&S.bar[1], kNS);
+        for (int i = 0; i < 2; i++) {
+            bar_init(&S.bar[i], kNS + 1);         // every staging thread, and one plain arrival
+            bar_init(&S.empty[i], kNC / 32);      // every sweeping warp
+        }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-        S.abort = 0;
-        S.pref = 0;
-        S.work = (long long)atomicAdd(&P.ctr->work_next, 1ull);
+        S.abort = S.late = 0;
+        S.work[0] = S.work[1] = 0;
     }
-    unsigned gb = 0;   // batches staged by this CTA before the current item (barrier phases)
-    unsigned ni = 0;   // items taken by this CTA (parity selects the run and row tables)
-    float msum = 0.0f, mcomp = 0.0f;  // Kahan-compensated FP32 mass of this thread
+    __syncthreads();
+    if (tid >= kNC) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsStage));
+        stage_loop<kA0X, kCodec>(P, S, tid - kNC, nbatch, nwork);
+        return;
+    }
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kRegsSweep));
+    unsigned gb = 0;                    // batches before the current item (barrier phases)
+    float msum = 0.0f, mcomp = 0.0f;    // Kahan-compensated FP32 mass of this thread
+    bool stop = false;
 
-    for (;; ni++) {
-        __syncthreads();
-        const int64_t w = S.work;
-        if (w >= nwork || S.abort) break;
-        const bool pref = S.pref != 0;
-        const int ti = (int)(ni & 1u);
-        const Item it = decode_item(P, w);
-        const int64_t okeep = (int64_t)P.out.base[it.b];
+    // a staged batch, or the end of the work list
+    auto wait_staged = [&](unsigned g) {
+        const unsigned slot = g & 1u, parity = (g >> 1) & 1u;
+        if (P.report_late && tid == 0 && !bar_test(&S.bar[slot], parity)) atomicOr(&P.ctr->error, 4);
+        if (!bar_wait_bounded(&S.bar[slot], parity)) {
+            atomicOr(&P.ctr->error, 4);
+            S.abort = 1;
+        }
+    };
+    for (int par = 0; !stop; par ^= 1) {
+        wait_staged(gb);
+        named_sync(kBarSweep, kNC);
+        if (S.abort || S.work[par] >= nwork) break;
+        const Item& it = S.item[par];
+        const ItemTables& tab = S.tab[par];
         using T = typename Codec<kCodec>::T;
-        T* opool = static_cast<T*>(P.out.pool);
-        if (!pref) item_tables(P, S, it, ti, tid);
-        if (tid < 3 * kChunk) {
-            // sweep constants of the item's 16 velocity cells (v = vx + 4 vy, vz = q)
-            const int j = tid >> 4, l = tid & 15;
-            const int d = P.ax[j];
-            const int bc = d == 0 ? it.b % G.nbx : (d == 1 ? (it.b / G.nbx) % G.nby : it.b / (G.nbx * G.nby));
-            const int wi = d == 0 ? (l & 3) : (d == 1 ? (l >> 2) : it.q);
-            S.kc[j][l] = P.walk[d * P.nvmax + bc * 4 + wi];
-        } else if (tid == 64) {
-            S.next = (long long)atomicAdd(&P.ctr->work_next, 1ull);
-        }
-        __syncthreads();  // per-item tables ready
-        if (tid == 0) {
-            S.pref = 0;
-            S.work = S.next;
-        }
-        const bool up0 = S.kc[0][0].w != 0.0f, up1 = S.kc[1][0].w != 0.0f;
-        auto out_of = [&](int s) { return it.up2 ? s - kFirst : n2 + 4 - s; };
-
+        const bool up0 = it.up0 != 0, up1 = it.up1 != 0, up2 = it.up2 != 0;
+        const bool dense_out = it.dense_out != 0;
         // ---- sweep-2 state of this thread: two tile cells, one vx row of the chunk ----
         const int zq = tid & 3;             // vy of the thread's vx row
-        const int zc = tid >> 2;            // tile cells zc and zc + 128
-        const int zcx = zc & 15, zcr = zc >> 4;
+        const int zcx = (tid >> 2) & 15, zcr = tid >> 6;  // tile cells (zcx, zcr) and (zcx, zcr + 8)
         const bool zv0 = zcx < it.ex && zcr < it.er, zv1 = zcx < it.ex && zcr + 8 < it.er;
         const int zoff = (kHalo + zcr) * kRP + (kHalo + zcx) * kChunk + 4 * zq;
-        const int64_t zcell = (int64_t)(it.tx0 + zcx) + (int64_t)(it.tr0 + zcr) * str_r;  // at plane 0
+        // dense next layout: the slot of the first cell in the plane that is emitted next
+        // (slots of one block id are below 2^31 like the cells)
+        unsigned zslot = (unsigned)(it.tx0 + zcx + (it.tr0 + zcr) * str_r + (up2 ? 0 : (n2 - 1) * str_2));
+        const unsigned zstep = up2 ? str_2 : -str_2;
+        T* const zpool = static_cast<T*>(P.out.pool) + it.obase + 4 * zq;
+        uint8_t* const kq = P.keepq + it.okeep * 4 + it.q;
+        float* const zscale = kCodec ? P.out.scale + it.obase / kChunk : nullptr;
+        // the four threads of a cell vote on its keep flag, which the first of them writes
+        // (nobody when none are wanted)
+        const unsigned vote = P.keepq && zq == 0 ? 0xfu << (lane & ~3) : 0u;
+        const float thr = P.thr;
         Walk2<kLim, 1> zw[4];
 #pragma unroll
         for (int i = 0; i < 4; i++) zw[i].reset();
-        const WalkConst2 kz = pack_const(S.kc[2][4 * zq], S.kc[2][4 * zq]);  // the streamed axis is not x: equal over vx
+        const WalkConst2 kz = pack_const(tab.kc[2][4 * zq], tab.kc[2][4 * zq]);  // the streamed axis is not x: equal over vx
 
-        if (stager && !pref) stage_batch<kCodec, kA0X>(P, S, it, ti, 0, gb, sl);
-        int k = 0;
-        for (; k < nbatch; k++) {
-            const unsigned slot = (gb + k) & 1u;
-            const unsigned parity = ((gb + k) >> 1) & 1u;
-            if (P.report_late && tid == 0 && !bar_test(&S.bar[slot], parity)) atomicOr(&P.ctr->error, 4);
-            if (!bar_wait_bounded(&S.bar[slot], parity)) {
-                atomicOr(&P.ctr->error, 4);
-                S.abort = 1;
-            }
+        for (int k = 0; k < nbatch; k++) {
+            const unsigned g = gb + (unsigned)k;
+            const unsigned slot = g & 1u;
+            if (k > 0) wait_staged(g);
             float* B = S.buf[slot][0];
             const int nj = min(kNB, nsteps - kNB * k);
             // sweep 0 along axis 0 on the halo lines that sweep 1 reads
@@ -604,7 +693,7 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
                 const int j = tid / (kLines * 8), rem = tid - j * (kLines * 8);
                 const int line = rem >> 3, l0 = 2 * (rem & 7);
                 if (j < nj) {
-                    const WalkConst2 kx = pack_const(S.kc[0][l0], S.kc[0][l0 + 1]);
+                    const WalkConst2 kx = pack_const(tab.kc[0][l0], tab.kc[0][l0 + 1]);
                     float* p = B + j * kPS + (line + (up1 ? 0 : 1)) * kS1 + l0;
                     // 16-bit storage: chunk scales of the line's cells
                     const float* ps = scales_of(S) + (slot * kNB + j) * kE * kSP + (line + (up1 ? 0 : 1)) * kC1;
@@ -641,28 +730,17 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
                     }
                 }
             }
-            __syncthreads();  // sweep 0 complete; the buffer of batch k-1 is free
-            if (S.abort) break;
-            if (stager) {
-                if (k + 1 < nbatch) {
-                    stage_batch<kCodec, kA0X>(P, S, it, ti, k + 1, gb + k + 1, sl);
-                } else {
-                    // last batch: stage the first batch of the next item
-                    const int64_t wn = S.next;
-                    if (wn < nwork) {
-                        const Item nx = decode_item(P, wn);
-                        item_tables(P, S, nx, ti ^ 1, tid);
-                        asm volatile("bar.sync 1, %0;\n" ::"n"(kNS) : "memory");
-                        stage_batch<kCodec, kA0X>(P, S, nx, ti ^ 1, 0, gb + nbatch, sl);
-                        if (sl == 0) S.pref = 1;
-                    }
-                }
-            } else {
+            named_sync(kBarSweep, kNC);  // sweep 0 complete
+            if (S.abort) {
+                stop = true;
+                break;
+            }
+            if (tid < kNY) {
                 // sweep 1 along axis 1 on the tile lines
                 const int j = tid >> 7, rem = tid & 127;
                 const int line = rem >> 3, l0 = 2 * (rem & 7);
                 if (j < nj) {
-                    const WalkConst2 ky = pack_const(S.kc[1][l0], S.kc[1][l0 + 1]);
+                    const WalkConst2 ky = pack_const(tab.kc[1][l0], tab.kc[1][l0 + 1]);
                     float* p = B + j * kPS + (kHalo + line) * kS0 + l0;
                     Walk2<kLim, 1> wk;
                     wk.reset();
@@ -684,82 +762,65 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
             // the in-place writes of this batch precede the bulk copies that refill the
             // buffer two batches on
             fence_async_smem();
-            // sweep 1 complete.  The sweep-1 warps do not wait for the staging warps, whose
-            // bulk-copy issue can outlast sweep 1: they arrive on barrier 2 and wait among
-            // themselves (barrier 3); the staging warps wait on barrier 2 for them
-            if (stager) {
-                asm volatile("bar.sync 2, %0;\n" ::"n"(kNC) : "memory");
-            } else {
-                asm volatile("bar.arrive 2, %0;\n" ::"n"(kNC) : "memory");
-                asm volatile("bar.sync 3, %0;\n" ::"n"(kNY) : "memory");
-            }
+            named_sync(kBarSweep, kNC);  // sweep 1 complete
             // sweep 2: push the batch's planes through the streamed windows and emit
             auto zplane = [&](int j) {
                 const int s = kNB * k + j;
                 const float* src = B + j * kPS + zoff;
                 const float4 y0 = *reinterpret_cast<const float4*>(src);
                 const float4 y1 = *reinterpret_cast<const float4*>(src + 8 * kRP);
-                const float2 r00 = zw[0].push(make_float2(y0.x, y0.y), kz);
-                const float2 r01 = zw[1].push(make_float2(y0.z, y0.w), kz);
-                const float2 r10 = zw[2].push(make_float2(y1.x, y1.y), kz);
-                const float2 r11 = zw[3].push(make_float2(y1.z, y1.w), kz);
+                float2 v[4];
+                v[0] = zw[0].push(make_float2(y0.x, y0.y), kz);
+                v[1] = zw[1].push(make_float2(y0.z, y0.w), kz);
+                v[2] = zw[2].push(make_float2(y1.x, y1.y), kz);
+                v[3] = zw[3].push(make_float2(y1.z, y1.w), kz);
                 if (s < kFirst) return;
-                const int zo = out_of(s);
-                int64_t rk0, rk1;
-                if (it.dense_out) {
-                    const int64_t c = zcell + (int64_t)zo * str_2;
-                    rk0 = zv0 ? c : -1;
-                    rk1 = zv1 ? c + 8 * str_r : -1;
+                // slots of the two cells (-1: none): in a dense next layout the cell index
+                int r0 = -1, r1 = -1;
+                if (dense_out) {
+                    r0 = zv0 ? (int)zslot : -1;
+                    r1 = zv1 ? (int)(zslot + zrow8) : -1;
+                    zslot += zstep;
                 } else {
-                    const int* orow = &S.orank[slot][j][0];
-                    rk0 = zv0 ? orow[zc] : -1;
-                    rk1 = zv1 ? orow[zc + 128] : -1;
+                    const int* orow = &S.orank[slot][j][zcr * kT + zcx];
+                    r0 = zv0 ? orow[0] : -1;
+                    r1 = zv1 ? orow[8 * kT] : -1;
                 }
                 float psum = 0.0f;
-                bool keep0 = false, keep1 = false;
-                // 16-bit storage: the scale of each of the two cells' chunk, from the largest
-                // magnitude over the four threads (vx rows) of the cell
+                // 16-bit storage: the scales of the two cells' chunks, from the largest magnitude
+                // over the four threads (vx rows) of a cell
                 ChunkScale cs0{1.0f, 1.0f}, cs1{1.0f, 1.0f};
                 if constexpr (kCodec != 0) {
-                    cs0 = chunk_scale(group_max<4>(
-                        fmaxf(fmaxf(fabsf(r00.x), fabsf(r00.y)), fmaxf(fabsf(r01.x), fabsf(r01.y)))));
-                    cs1 = chunk_scale(group_max<4>(
-                        fmaxf(fmaxf(fabsf(r10.x), fabsf(r10.y)), fmaxf(fabsf(r11.x), fabsf(r11.y)))));
+                    auto top = [](const float2& p, const float2& q) {
+                        return fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fmaxf(fabsf(q.x), fabsf(q.y)));
+                    };
+                    cs0 = chunk_scale(group_max<4>(top(v[0], v[1])));
+                    cs1 = chunk_scale(group_max<4>(top(v[2], v[3])));
                 }
-                // store one vx row (4 values) of a cell; v0, v1 become the values the state
-                // now holds (16-bit storage: the codes decoded)
-                auto store = [&](int64_t rk, float2& v0, float2& v1, const ChunkScale& cs) {
-                    T* dst = opool + it.obase + rk * kChunk + 4 * zq;
+                // one vx row (4 values) of a cell; the values summed and compared are those that
+                // the state now holds (16-bit storage: the codes decoded).  No branches: the
+                // stores are predicated
+                auto emit = [&](int r, float2 v0, float2 v1, const ChunkScale& cs) -> bool {
+                    const bool has = r >= 0;
+                    T* dst = zpool + (int64_t)r * kChunk;
                     if constexpr (kCodec == 0) {
-                        *reinterpret_cast<float4*>(dst) = make_float4(v0.x, v0.y, v1.x, v1.y);
+                        if (has) *reinterpret_cast<float4*>(dst) = make_float4(v0.x, v0.y, v1.x, v1.y);
                     } else {
                         const float2 inv = make_float2(cs.inv, cs.inv), sc = make_float2(cs.s, cs.s);
                         const uint32_t w0 = enc2<kCodec>(v0, inv), w1 = enc2<kCodec>(v1, inv);
-                        *reinterpret_cast<uint2*>(dst) = make_uint2(w0, w1);
-                        if (zq == 0) P.out.scale[it.obase / kChunk + rk] = cs.s;
+                        if (has) *reinterpret_cast<uint2*>(dst) = make_uint2(w0, w1);
+                        if (has && zq == 0) zscale[r] = cs.s;
                         v0 = dec2<kCodec>(w0, sc);
                         v1 = dec2<kCodec>(w1, sc);
                     }
+                    psum += has ? (v0.x + v0.y) + (v1.x + v1.y) : 0.0f;
+                    return has && fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)) >= thr;
                 };
-                if (rk0 >= 0) {
-                    float2 v0 = r00, v1 = r01;
-                    store(rk0, v0, v1, cs0);
-                    psum += (v0.x + v0.y) + (v1.x + v1.y);
-                    keep0 = fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)) >= P.thr;
-                }
-                if (rk1 >= 0) {
-                    float2 v0 = r10, v1 = r11;
-                    store(rk1, v0, v1, cs1);
-                    psum += (v0.x + v0.y) + (v1.x + v1.y);
-                    keep1 = fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)) >= P.thr;
-                }
+                const bool keep0 = emit(r0, v[0], v[1], cs0), keep1 = emit(r1, v[2], v[3], cs1);
                 // per-chunk keep flags: the four threads of a cell vote
-                const unsigned b0 = __ballot_sync(0xffffffffu, keep0);
-                const unsigned b1 = __ballot_sync(0xffffffffu, keep1);
-                if (zq == 0) {
-                    if ((b0 >> (lane & ~3)) & 0xfu) P.keepq[(okeep + rk0) * 4 + it.q] = 1;
-                    if ((b1 >> (lane & ~3)) & 0xfu) P.keepq[(okeep + rk1) * 4 + it.q] = 1;
-                }
+                const unsigned b0 = __ballot_sync(0xffffffffu, keep0), b1 = __ballot_sync(0xffffffffu, keep1);
+                if (b0 & vote) kq[(int64_t)r0 * 4] = 1;
+                if (b1 & vote) kq[(int64_t)r1 * 4] = 1;
                 const float y = psum - mcomp;
                 const float t = msum + y;
                 mcomp = (t - msum) - y;
@@ -771,19 +832,15 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
             } else {
                 for (int j = 0; j < nj; j++) zplane(j);
             }
-        }
-        if (S.abort) {
-            // leave no bulk copy in flight: the batch whose wait ran out is the only one
-            // staged and not yet complete
-            if (tid == 0 && k < nbatch) bar_wait_bounded(&S.bar[(gb + k) & 1u], ((gb + k) >> 1) & 1u);
-            break;
+            // this warp has read the buffer
+            __syncwarp();
+            if (lane == 0) bar_arrive(&S.empty[slot]);
         }
         gb += (unsigned)nbatch;
     }
     double m = (double)msum;
     for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
     if (lane == 0 && m != 0.0) atomicAdd(&P.ctr->mass, m);
-    __syncthreads();
     if (P.cta_done && tid == 0) P.cta_done[blockIdx.x] = now_ns();
 }
 
@@ -791,6 +848,11 @@ template <bool kLim, bool kA0X, int kCodec>
 vl_status launch_gt3(Grid* g, const Gt3Args& P)
 {
     auto kern = k_gt3<kLim, kA0X, kCodec>;
+    // setmaxnreg draws on the registers of the launch: never start a kernel whose share
+    // is smaller than the split
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.numRegs * kNT < kNC * kRegsSweep + kNS * kRegsStage)
+        return fail(g, VL_ECUDA, "plane-batched fused sweep: register count of the kernel");
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<kCodec>());
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->dev.device);
@@ -852,7 +914,7 @@ vl_status run_gt3(Grid* g, const StepArgs& a)
     T.ntile0 = ntile0;
     T.ntile1 = ntile1;
     T.ty = kT;
-    launch_tile_list(g, T, need, ntiles);
+    launch_tile_list(g, T, need, ntiles, true);
 
     Gt3Args P;
     P.G = G;
@@ -867,8 +929,9 @@ vl_status run_gt3(Grid* g, const StepArgs& a)
     P.nvmax = a.nvmax;
     P.thr = (float)g->threshold;
     P.ntile0 = ntile0;
+    P.ntiles = (uint32_t)ntiles;
     P.items = g->items;
-    P.item_base = g->item_base;
+    P.npairs = g->item_base + G.nb;
     P.keepq = B.keepq;
     P.ctr = a.ctr;
     P.report_late = fault_requested("timeout") ? 1 : 0;
