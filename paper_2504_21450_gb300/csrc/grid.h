@@ -202,6 +202,11 @@ void launch_tile_list(Grid* g, const TileArgs& T, int64_t need, int64_t ntiles, 
 // gt3.cu: the plane-batched GT3 kernel (GT3, streamed axis y or z, no
 // velocity block straddling v_d = 0)
 bool gt3_applies(const Grid* g, const StepArgs& a);
+bool gt3_fits(const vl_vmesh_desc& vmesh, const double c_scale[3], const int order[3]);
+int64_t gt3_tiles(const GridGeom& G, const int order[3]);  // tiles per block id
+vl_status launch_gt3_dense(const GridGeom& G, const LayoutView& in, const LayoutView& out, const int order[3],
+                           int limiter, const float4* ctab, int nvmax, const uint32_t* items,
+                           const int64_t* npairs, StepCounters* ctr, int device, cudaStream_t stream);
 vl_status run_gt3(Grid* g, const StepArgs& a);
 inline bool use_gt3(const Grid* g, const StepArgs& a)
 {

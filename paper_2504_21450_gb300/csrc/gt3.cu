@@ -867,28 +867,63 @@ vl_status launch_gt3(Grid* g, const Gt3Args& P)
     return VL_OK;
 }
 
-inline int nblocks_of(int64_t n, int t) { return (int)((n + t - 1) / t); }
-
 }  // namespace
 
-bool gt3_applies(const Grid* g, const StepArgs& a)
+bool gt3_fits(const vl_vmesh_desc& vmesh, const double c_scale[3], const int order[3])
 {
-    if (a.ghost != 3) return false;
-    if (a.order[2] == 0) return false;  // streamed axis must not be x
+    if (order[2] == 0) return false;  // streamed axis must not be x
     // every velocity block moves one way along each axis
     for (int d = 0; d < 3; d++)
-        for (int bi = 0; bi < g->vmesh.nv[d] / 4; bi++) {
-            const double lo = g->vmesh.vmin[d] + (4 * bi + 0.5) * g->vmesh.dv[d];
-            const double hi = g->vmesh.vmin[d] + (4 * bi + 3.5) * g->vmesh.dv[d];
-            if ((lo * a.c_scale[d] >= 0.0) != (hi * a.c_scale[d] >= 0.0)) return false;
+        for (int bi = 0; bi < vmesh.nv[d] / 4; bi++) {
+            const double lo = vmesh.vmin[d] + (4 * bi + 0.5) * vmesh.dv[d];
+            const double hi = vmesh.vmin[d] + (4 * bi + 3.5) * vmesh.dv[d];
+            if ((lo * c_scale[d] >= 0.0) != (hi * c_scale[d] >= 0.0)) return false;
         }
     return true;
 }
 
-int64_t gt3_tiles(const Grid* g, const StepArgs& a)
+bool gt3_applies(const Grid* g, const StepArgs& a)
 {
-    const int ar = a.order[0] == 0 ? a.order[1] : a.order[0];
-    return (int64_t)((g->geom.n[0] + kT - 1) / kT) * ((g->geom.n[ar] + kT - 1) / kT);
+    return a.ghost == 3 && gt3_fits(g->vmesh, a.c_scale, a.order);
+}
+
+int64_t gt3_tiles(const GridGeom& G, const int order[3])
+{
+    const int ar = order[0] == 0 ? order[1] : order[0];
+    return (int64_t)((G.n[0] + kT - 1) / kT) * ((G.n[ar] + kT - 1) / kT);
+}
+
+// One launch over caller-provided buffers of a dense FP32 layout: items are all nb * tiles
+// pairs in order, npairs their number, no keep flags (the caller's threshold is +inf).
+vl_status launch_gt3_dense(const GridGeom& G, const LayoutView& in, const LayoutView& out, const int order[3],
+                           int limiter, const float4* ctab, int nvmax, const uint32_t* items,
+                           const int64_t* npairs, StepCounters* ctr, int device, cudaStream_t stream)
+{
+    Gt3Args P;
+    P.G = G;
+    P.in = in;
+    P.out = out;
+    for (int j = 0; j < 3; j++) P.ax[j] = order[j];
+    P.ar = order[0] == 0 ? order[1] : order[0];
+    P.stride[0] = 1;
+    P.stride[1] = G.n[0];
+    P.stride[2] = (int64_t)G.n[0] * G.n[1];
+    P.walk = ctab;
+    P.nvmax = nvmax;
+    P.thr = INFINITY;
+    P.ntile0 = (G.n[0] + kT - 1) / kT;
+    P.ntiles = (uint32_t)gt3_tiles(G, order);
+    P.items = items;
+    P.npairs = npairs;
+    P.keepq = nullptr;
+    P.ctr = ctr;
+    P.report_late = 0;
+    P.cta_done = nullptr;
+    Grid tmp;  // launch helper needs the device and the stream only
+    tmp.dev.device = device;
+    tmp.stream = stream;
+    if (order[0] == 0) return limiter ? launch_gt3<true, true, 0>(&tmp, P) : launch_gt3<false, true, 0>(&tmp, P);
+    return limiter ? launch_gt3<true, false, 0>(&tmp, P) : launch_gt3<false, false, 0>(&tmp, P);
 }
 
 vl_status run_gt3(Grid* g, const StepArgs& a)
@@ -945,7 +980,6 @@ vl_status run_gt3(Grid* g, const StepArgs& a)
         else st = a.limiter ? launch_gt3<true, false, kc>(g, P) : launch_gt3<false, false, kc>(g, P);
     });
     record_sweep_event(a.ev1, g->stream, a.ev_node);
-    (void)nblocks_of;
     return st;
 }
 
