@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "grid.h"
@@ -40,96 +41,14 @@ struct TileGeom {
     int nt[3];  // tiles per dimension
 };
 
-// Velocity moments of every cell for the features: one warp per 64-cell bitmap word (a
-// row segment), looping over the block ids with one broadcast bitmap load each; a lane
-// owns cells x and x+32 of the word.  Each present block is summed in FP32 about its own
-// velocity centre v_b (offsets delta within +-1.5 dv: a = sum f, e_d = sum delta_d f,
-// q_d = sum delta_d^2 f), then per cell in FP64: n = sum a, nV_d = sum (v_b,d a + e_d),
-// S_d = sum (v_b,d^2 a + 2 v_b,d e_d + q_d), P_dd = S_d - (nV_d)^2 / n, all times dv^3.
-// The error of P is then relative to P itself (the rounding of a block's sums enters
-// with weight (v_b - V)^2), not to the much larger sum of v^2 f.
-struct VMeshF {
-    double vmin[3], dv[3];
-};
-
-template <int kCodec>
-__global__ void __launch_bounds__(256) k_cell_moments(GridGeom G, LayoutView L, VMeshF V, double* __restrict__ mom)
-{
-    using C = Codec<kCodec>;
-    using T = typename C::T;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (wid >= G.RW) return;  // warp-uniform
-    const int lane = threadIdx.x & 31;
-    const int64_t row = wid / G.W;
-    const int w = (int)(wid - row * G.W);
-    double A[2] = {0, 0}, B[2][3] = {{0, 0, 0}, {0, 0, 0}}, S[2][3] = {{0, 0, 0}, {0, 0, 0}};
-    const T* pool = static_cast<const T*>(L.pool);
-    for (int b = 0; b < G.nb; b++) {
-        const int64_t wi = (int64_t)b * G.RW + wid;
-        const uint64_t k = L.kbits[wi];
-        if (!k) continue;
-        const uint64_t u = L.ubits[wi];
-        const int64_t wo = L.woff[wi];
-        const int64_t base = L.base[b];
-        const int64_t cnt = L.cnt[b];
-        const bool dense = (L.dense[b] & 1) != 0;
-        const int bc[3] = {b % G.nbx, (b / G.nbx) % G.nby, b / (G.nbx * G.nby)};
-        double vb[3];
-        for (int d = 0; d < 3; d++) vb[d] = V.vmin[d] + (4 * bc[d] + 2) * V.dv[d];
-        const float dvx = (float)V.dv[0], dvy = (float)V.dv[1], dvz = (float)V.dv[2];
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int bit = lane + 32 * h;
-            if (!((k >> bit) & 1ull)) continue;
-            const int64_t rank = dense ? row * G.n[0] + 64 * w + bit : wo + __popcll(u & ((1ull << bit) - 1ull));
-            float a = 0.f, e[3] = {0.f, 0.f, 0.f}, q[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-            for (int iz = 0; iz < 4; iz++) {
-                const int64_t chunk = base * 4 + iz * cnt + rank;
-                const T* src = pool + chunk * kChunk;
-                const float sc = kCodec ? L.scale[chunk] : 1.0f;
-                const float dz = (iz - 1.5f) * dvz;
-#pragma unroll
-                for (int l = 0; l < kChunk; l++) {
-                    const float f = C::dec(src[l], sc);
-                    const float dx = ((l & 3) - 1.5f) * dvx, dy = ((l >> 2) - 1.5f) * dvy;
-                    a += f;
-                    e[0] = fmaf(dx, f, e[0]);
-                    e[1] = fmaf(dy, f, e[1]);
-                    e[2] = fmaf(dz, f, e[2]);
-                    q[0] = fmaf(dx * dx, f, q[0]);
-                    q[1] = fmaf(dy * dy, f, q[1]);
-                    q[2] = fmaf(dz * dz, f, q[2]);
-                }
-            }
-            A[h] += a;
-            for (int d = 0; d < 3; d++) {
-                B[h][d] += vb[d] * a + e[d];
-                S[h][d] += vb[d] * vb[d] * a + 2.0 * vb[d] * e[d] + q[d];
-            }
-        }
-    }
-    const double dv3 = V.dv[0] * V.dv[1] * V.dv[2];
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int x = 64 * w + lane + 32 * h;
-        if (x >= G.n[0]) continue;
-        double* o = mom + (row * G.n[0] + x) * 7;
-        o[0] = A[h] * dv3;
-        for (int d = 0; d < 3; d++) {
-            o[1 + d] = B[h][d] * dv3;
-            o[4 + d] = A[h] != 0.0 ? (S[h][d] - B[h][d] * B[h][d] / A[h]) * dv3 : 0.0;
-        }
-    }
-}
-
-// Per tile: active blocks (kbits of the state), blocks of the next step's union (ubits
-// of the next layout), and FP64 sums over the tile's cells of n, V_d, v_th and the
-// relative density gradient, from the per-cell moments (n, nV_d, P_dd).
-__global__ void __launch_bounds__(256) k_tile_features(TileGeom T, const uint64_t* __restrict__ kbits,
-                                                       const uint64_t* __restrict__ ubits,
-                                                       const double* __restrict__ mom,
-                                                       float* __restrict__ feat, float* __restrict__ uni)
+// Per tile: active blocks (kbits of the state) and blocks of the next step's union (ubits
+// of the next layout), counts[tile] = {active, union}.  A CTA takes a tile and a part of the
+// block ids, so that a few hundred tiles still fill the chip (one CTA per tile took 0.80 ms
+// on 216 tiles x 4096 ids, 0.14 with the ids split); integer sums, so their order does
+// not matter.
+__global__ void __launch_bounds__(256) k_tile_counts(TileGeom T, int ids, const uint64_t* __restrict__ kbits,
+                                                     const uint64_t* __restrict__ ubits,
+                                                     unsigned long long* __restrict__ counts)
 {
     const GridGeom& G = T.G;
     const int tile = blockIdx.x;
@@ -139,13 +58,13 @@ __global__ void __launch_bounds__(256) k_tile_features(TileGeom T, const uint64_
         lo[d] = tc[d] * T.edge;
         ext[d] = min(T.edge, G.n[d] - lo[d]);
     }
-    // block counts: (block id, tile row) pairs, the tile's x range masked in each word
+    // (block id, tile row) pairs, the tile's x range masked in each word
     const int rows = ext[1] * ext[2];
-    const int64_t pairs = (int64_t)G.nb * rows;
-    unsigned long long act = 0, un = 0;
-    for (int64_t i = threadIdx.x; i < pairs; i += blockDim.x) {
-        const int b = (int)(i / rows);
-        const int r = (int)(i - (int64_t)b * rows);
+    const int b0 = blockIdx.y * ids, b1 = min(G.nb, b0 + ids);
+    unsigned act = 0, un = 0;
+    for (int i = threadIdx.x; i < (b1 - b0) * rows; i += blockDim.x) {
+        const int b = b0 + i / rows;
+        const int r = i % rows;
         const int64_t row = (int64_t)(lo[1] + r % ext[1]) + (int64_t)G.n[1] * (lo[2] + r / ext[1]);
         const int64_t base = (int64_t)b * G.RW + row * G.W;
         for (int x = lo[0]; x < lo[0] + ext[0];) {  // words overlapping the x range
@@ -157,6 +76,28 @@ __global__ void __launch_bounds__(256) k_tile_features(TileGeom T, const uint64_
             un += __popcll(ubits[base + w] & m);
             x = xe;
         }
+    }
+    act = __reduce_add_sync(0xffffffffu, act);
+    un = __reduce_add_sync(0xffffffffu, un);
+    if ((threadIdx.x & 31) == 0) {
+        if (act) atomicAdd(&counts[2 * tile], (unsigned long long)act);
+        if (un) atomicAdd(&counts[2 * tile + 1], (unsigned long long)un);
+    }
+}
+
+// Per tile: its block counts, and FP64 sums over the tile's cells of n, V_d, v_th and the
+// relative density gradient, from the per-cell moments (n, nV_d, P_dd).
+__global__ void __launch_bounds__(256) k_tile_features(TileGeom T, const unsigned long long* __restrict__ counts,
+                                                       const double* __restrict__ mom,
+                                                       float* __restrict__ feat, float* __restrict__ uni)
+{
+    const GridGeom& G = T.G;
+    const int tile = blockIdx.x;
+    const int tc[3] = {tile % T.nt[0], (tile / T.nt[0]) % T.nt[1], tile / (T.nt[0] * T.nt[1])};
+    int lo[3], ext[3];
+    for (int d = 0; d < 3; d++) {
+        lo[d] = tc[d] * T.edge;
+        ext[d] = min(T.edge, G.n[d] - lo[d]);
     }
     // per-cell moment features
     double s[6] = {0, 0, 0, 0, 0, 0};  // n, Vx, Vy, Vz, v_th, and (max) |grad n| / n
@@ -186,28 +127,20 @@ __global__ void __launch_bounds__(256) k_tile_features(TileGeom T, const uint64_
     }
     // deterministic CTA reduction: warp trees, then warps in order
     __shared__ double sh[8][6];
-    __shared__ unsigned long long shc[8][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int o = 16; o > 0; o >>= 1) {
         for (int k = 0; k < 5; k++) s[k] += __shfl_down_sync(0xffffffffu, s[k], o);
         s[5] = fmax(s[5], __shfl_down_sync(0xffffffffu, s[5], o));
-        act += __shfl_down_sync(0xffffffffu, act, o);
-        un += __shfl_down_sync(0xffffffffu, un, o);
     }
-    if (lane == 0) {
+    if (lane == 0)
         for (int k = 0; k < 6; k++) sh[warp][k] = s[k];
-        shc[warp][0] = act;
-        shc[warp][1] = un;
-    }
     __syncthreads();
     if (threadIdx.x == 0) {
         double t[6] = {0, 0, 0, 0, 0, 0};
-        unsigned long long A = 0, U = 0;
+        const unsigned long long A = counts[2 * tile], U = counts[2 * tile + 1];
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
             for (int k = 0; k < 5; k++) t[k] += sh[w][k];
             t[5] = fmax(t[5], sh[w][5]);
-            A += shc[w][0];
-            U += shc[w][1];
         }
         float* f = feat + (int64_t)tile * kIn;
         f[0] = (float)log1p((double)A);
@@ -425,33 +358,40 @@ vl_status tile_features(Grid* g, int edge, float* feat, float* uni)
     const GridGeom& G = g->geom;
     if (edge < 1 || edge > 64 || !feat || !uni) return fail(g, VL_EINVAL, "vl_tile_features: bad arguments");
     if (!g->has_state) return fail(g, VL_ESTATE, "vl_tile_features: no state");
-    double* mom = (double*)g->alloc((size_t)G.N * 7 * 8);
-    if (!mom) return fail(g, VL_ENOMEM, "vl_tile_features: scratch allocation failed");
-    VMeshF V;
-    for (int d = 0; d < 3; d++) {
-        V.vmin[d] = g->vmesh.vmin[d];
-        V.dv[d] = g->vmesh.dv[d];
-    }
-    const Layout& Lc = g->lay[g->cur];
-    with_codec(g->codec, [&](auto c) {
-        k_cell_moments<decltype(c)::value><<<nblk(G.RW * 32, 256), 256, 0, g->stream>>>(G, Lc.view(), V, mom);
-    });
-    note_launch();
-    // the next layout's ubits become the 27-cell union of the state (the next step
-    // rebuilds that layout anyway)
-    launch_union(g, g->lay[g->cur], g->lay[1 - g->cur]);
+    int64_t ntiles = 1;
     TileGeom T;
     T.G = G;
     T.edge = edge;
-    int64_t ntiles = 1;
     for (int d = 0; d < 3; d++) {
         T.nt[d] = (G.n[d] + edge - 1) / edge;
         ntiles *= T.nt[d];
     }
-    k_tile_features<<<(unsigned)ntiles, 256, 0, g->stream>>>(T, g->lay[g->cur].kbits, g->lay[1 - g->cur].ubits,
-                                                             mom, feat, uni);
+    // per-cell moments, then the tiles' block counts
+    double* mom = (double*)g->alloc((size_t)G.N * 7 * 8 + (size_t)ntiles * 16);
+    if (!mom) return fail(g, VL_ENOMEM, "vl_tile_features: scratch allocation failed");
+    unsigned long long* counts = reinterpret_cast<unsigned long long*>(mom + G.N * 7);
+    cudaMemsetAsync(counts, 0, (size_t)ntiles * 16, g->stream);
+    void* parts = nullptr;
+    vl_status st = queue_cell_moments(g, mom, &parts);
+    if (st != VL_OK) {
+        cudaStreamSynchronize(g->stream);
+        g->release(parts);
+        g->release(mom);
+        return st;
+    }
+    // the next layout's ubits become the 27-cell union of the state (the next step
+    // rebuilds that layout anyway)
+    launch_union(g, g->lay[g->cur], g->lay[1 - g->cur]);
+    // about eight CTAs per SM, parts of at least 16 ids
+    const int split = (int)std::max<int64_t>(1, std::min<int64_t>((G.nb + 15) / 16, 152 * 8 / ntiles));
+    const int ids = (G.nb + split - 1) / split;
+    k_tile_counts<<<dim3((unsigned)ntiles, (unsigned)((G.nb + ids - 1) / ids)), 256, 0, g->stream>>>(
+        T, ids, g->lay[g->cur].kbits, g->lay[1 - g->cur].ubits, counts);
+    note_launch();
+    k_tile_features<<<(unsigned)ntiles, 256, 0, g->stream>>>(T, counts, mom, feat, uni);
     note_launch();
     cudaError_t e = cudaStreamSynchronize(g->stream);
+    g->release(parts);
     g->release(mom);
     return e == cudaSuccess ? VL_OK : cuda_fail(g, e, "vl_tile_features");
 }

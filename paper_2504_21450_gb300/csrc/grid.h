@@ -130,7 +130,15 @@ vl_status get_window(Grid* g, const int* origin, const int* size, int64_t capaci
                      int64_t* off_out, uint16_t* ids_out, float* vals_out, int on_device,
                      int64_t* count);
 vl_status moments(Grid* g, double* out, int on_device);
+// Queues the moments of every cell into d_out (device, [cells][7]); *scratch (or nullptr) is
+// released by the caller once the stream has passed.
+vl_status queue_cell_moments(Grid* g, double* d_out, void** scratch);
 vl_status tile_features(Grid* g, int edge, float* feat, float* uni);
+// ---- moments.cu ------------------------------------------------------------
+// The velocity mesh is narrow enough for queue_moments, which is queue_cell_moments for
+// such meshes.
+bool moments_fit(const Grid* g);
+vl_status queue_moments(Grid* g, double* d_out, void** scratch);
 vl_status total_mass(Grid* g, double* mass);
 // Generic scans used by the layout code and the work lists.
 void launch_seg_scan(const uint32_t* in, uint32_t* out, uint32_t* seg_total, int64_t seg_len,

@@ -429,7 +429,9 @@ __device__ __forceinline__ double warp_sum(double x)
     return x;
 }
 
-// One warp per cell; two passes over the cell's blocks (n and nV, then P about V).
+// Moments on velocity meshes too wide for the marginals of moments.cu (more than 1600
+// cells along the three axes together): one warp per cell, every value in FP64, two passes
+// over the cell's blocks (n and nV, then P about V).
 template <int kCodec>
 __global__ void k_moments(GridGeom G, LayoutView L, VMesh V, double* __restrict__ out)
 {
@@ -498,16 +500,6 @@ __global__ void k_popcount(const uint64_t* __restrict__ u, uint32_t* __restrict_
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) c[i] = (uint32_t)__popcll(u[i]);
-}
-
-__global__ void k_sum_density(const double* __restrict__ mom, int64_t N, double* __restrict__ out)
-{
-    double s = 0.0;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < N;
-         c += (int64_t)gridDim.x * blockDim.x)
-        s += mom[c * 7];
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
 
 inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
@@ -1075,46 +1067,38 @@ vl_status set_blocks_planes(Grid* g, int z0, int nplanes, int64_t Mw, const int6
     return set_blocks(g, M, off_n, ids_n, vals_n, 1);
 }
 
-vl_status moments(Grid* g, double* out, int on_device)
+vl_status queue_cell_moments(Grid* g, double* d_out, void** scratch)
 {
     const GridGeom& G = g->geom;
-    const Layout& L = g->lay[g->cur];
-    if (!out) return fail(g, VL_EINVAL, "vl_moments: null pointer");
-    Scratch sc(g);
-    double* d_out = on_device ? out : (double*)sc.get((size_t)G.N * 7 * 8);
-    if (!d_out) return fail(g, VL_ENOMEM, "vl_moments: scratch allocation failed");
+    *scratch = nullptr;
+    if (moments_fit(g)) return queue_moments(g, d_out, scratch);
     VMesh V;
     for (int d = 0; d < 3; d++) {
         V.vmin[d] = g->vmesh.vmin[d];
         V.dv[d] = g->vmesh.dv[d];
     }
     with_codec(g->codec, [&](auto c) {
-        k_moments<decltype(c)::value><<<nblk(G.N * 32, 256), 256, 0, g->stream>>>(G, L.view(), V, d_out);
+        k_moments<decltype(c)::value><<<nblk(G.N * 32, 256), 256, 0, g->stream>>>(G, g->lay[g->cur].view(), V, d_out);
     });
     note_launch();
+    return VL_OK;
+}
+
+vl_status moments(Grid* g, double* out, int on_device)
+{
+    const GridGeom& G = g->geom;
+    if (!out) return fail(g, VL_EINVAL, "vl_moments: null pointer");
+    Scratch sc(g);
+    double* d_out = on_device ? out : (double*)sc.get((size_t)G.N * 7 * 8);
+    if (!d_out) return fail(g, VL_ENOMEM, "vl_moments: scratch allocation failed");
+    void* parts = nullptr;
+    vl_status st = queue_cell_moments(g, d_out, &parts);
+    if (parts) sc.ptrs.push_back(parts);
+    if (st != VL_OK) return st;
     if (!on_device)
         cudaMemcpyAsync(out, d_out, (size_t)G.N * 7 * 8, cudaMemcpyDeviceToHost, g->stream);
     cudaError_t e = cudaStreamSynchronize(g->stream);
     if (e != cudaSuccess) return cuda_fail(g, e, "vl_moments");
-    return VL_OK;
-}
-
-vl_status total_mass(Grid* g, double* mass)
-{
-    const GridGeom& G = g->geom;
-    Scratch sc(g);
-    double* mom = (double*)sc.get((size_t)G.N * 7 * 8);
-    double* acc = (double*)sc.get(8);
-    if (!mom || !acc) return fail(g, VL_ENOMEM, "vl_mass: scratch allocation failed");
-    vl_status st = moments(g, mom, 1);
-    if (st != VL_OK) return st;
-    cudaMemsetAsync(acc, 0, 8, g->stream);
-    k_sum_density<<<152 * 4, 256, 0, g->stream>>>(mom, G.N, acc); note_launch();
-    double h = 0.0;
-    cudaMemcpyAsync(&h, acc, 8, cudaMemcpyDeviceToHost, g->stream);
-    cudaError_t e = cudaStreamSynchronize(g->stream);
-    if (e != cudaSuccess) return cuda_fail(g, e, "vl_mass");
-    *mass = h * g->space.dx[0] * g->space.dx[1] * g->space.dx[2];
     return VL_OK;
 }
 
