@@ -168,139 +168,261 @@ __global__ void k_cost_targets(const float* __restrict__ trace, int nsnap, int64
 }
 
 // ---- MLP -----------------------------------------------------------------------------
-__device__ __forceinline__ void load_params(const float* __restrict__ params, float* sp)
+// A CTA of 512 threads works on batches of 16 samples with the parameters and the batch's
+// activations in shared memory.  In a layer a thread owns one unit and two samples, so that
+// a weight is read once for both; every dot product runs in the order of its index, so
+// an output does not depend on the batch it is in.
+constexpr int kMlpThreads = 512;
+constexpr int kMlpBatch = 16;
+constexpr int kPad = kH + 1;  // row pitch of W2: both its rows and its columns are read by a warp
+
+struct MlpSmem {
+    float w1[kH][kIn + 1], w2[kH][kPad];
+    float b1[kH], b2[kH], w3[kH], b3;
+    alignas(16) float x[kMlpBatch][kIn];
+    alignas(16) float h1[kMlpBatch][kH], h2[kMlpBatch][kH], d1[kMlpBatch][kH], d2[kMlpBatch][kH];
+    float y[kMlpBatch], dy[kMlpBatch];
+};
+
+__device__ __forceinline__ void load_params(const float* __restrict__ params, MlpSmem& S)
 {
-    for (int i = threadIdx.x; i < kP; i += blockDim.x) sp[i] = params[i];
+    for (int i = threadIdx.x; i < kP; i += blockDim.x) {
+        const float v = params[i];
+        if (i < ob1) S.w1[i / kIn][i % kIn] = v;
+        else if (i < oW2) S.b1[i - ob1] = v;
+        else if (i < ob2) S.w2[(i - oW2) / kH][(i - oW2) % kH] = v;
+        else if (i < ow3) S.b2[i - ob2] = v;
+        else if (i < ob3) S.w3[i - ow3] = v;
+        else S.b3 = v;
+    }
+}
+
+// Forward pass of samples s0 .. s0+m-1 (m <= kMlpBatch): y = b3 + w3 . relu(W2 relu(W1 x +
+// b1) + b2).  Ends with a barrier.
+__device__ __forceinline__ void forward_batch(MlpSmem& S, const float* __restrict__ x, int64_t s0, int m)
+{
+    const int tid = threadIdx.x, u = tid & (kH - 1), a = 2 * (tid / kH), b = a + 1;
+    if (tid < kMlpBatch * kIn) S.x[tid / kIn][tid % kIn] = tid / kIn < m ? x[s0 * kIn + tid] : 0.0f;
     __syncthreads();
-}
-
-// One thread per sample: y = b3 + w3 . relu(W2 relu(W1 x + b1) + b2); the hidden
-// activations are kept when h1/h2 are given (training).
-__global__ void __launch_bounds__(kThreads) k_mlp_forward(const float* __restrict__ params,
-                                                          const float* __restrict__ x, int64_t n,
-                                                          float* __restrict__ y, float* __restrict__ h1o,
-                                                          float* __restrict__ h2o)
-{
-    __shared__ float sp[kP];
-    load_params(params, sp);
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    float xi[kIn];
+    {
+        float p = S.b1[u], q = p;
 #pragma unroll
-    for (int i = 0; i < kIn; i++) xi[i] = x[s * kIn + i];
-    float h1[kH];
-#pragma unroll
-    for (int k = 0; k < kH; k++) {
-        float a = sp[ob1 + k];
-#pragma unroll
-        for (int i = 0; i < kIn; i++) a = fmaf(sp[oW1 + k * kIn + i], xi[i], a);
-        h1[k] = fmaxf(a, 0.0f);
-        if (h1o) h1o[s * kH + k] = h1[k];
-    }
-    float out = sp[ob3];
-    for (int j = 0; j < kH; j++) {
-        float a = sp[ob2 + j];
-#pragma unroll
-        for (int k = 0; k < kH; k++) a = fmaf(sp[oW2 + j * kH + k], h1[k], a);
-        const float h = fmaxf(a, 0.0f);
-        if (h2o) h2o[s * kH + j] = h;
-        out = fmaf(sp[ow3 + j], h, out);
-    }
-    y[s] = out;
-}
-
-// One thread per sample, loss L = (1/n) sum (y - t)^2: dL/dy, dL/d(pre-activation) of
-// layer 2 (dh2) and of layer 1 (dh1); the ReLU passes the gradient where its output > 0.
-__global__ void __launch_bounds__(kThreads) k_mlp_backward(const float* __restrict__ params,
-                                                           const float* __restrict__ y,
-                                                           const float* __restrict__ t, int64_t n,
-                                                           const float* __restrict__ h1,
-                                                           const float* __restrict__ h2,
-                                                           float* __restrict__ dy, float* __restrict__ dh1,
-                                                           float* __restrict__ dh2)
-{
-    __shared__ float sp[kP];
-    load_params(params, sp);
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const float g = 2.0f * (y[s] - t[s]) / (float)n;
-    dy[s] = g;
-    float d2[kH];
-#pragma unroll
-    for (int j = 0; j < kH; j++) {
-        d2[j] = h2[s * kH + j] > 0.0f ? g * sp[ow3 + j] : 0.0f;
-        dh2[s * kH + j] = d2[j];
-    }
-    for (int k = 0; k < kH; k++) {
-        float a = 0.0f;
-        if (h1[s * kH + k] > 0.0f) {
-#pragma unroll
-            for (int j = 0; j < kH; j++) a = fmaf(sp[oW2 + j * kH + k], d2[j], a);
+        for (int i = 0; i < kIn; i++) {
+            const float w = S.w1[u][i];
+            p = fmaf(w, S.x[a][i], p);
+            q = fmaf(w, S.x[b][i], q);
         }
-        dh1[s * kH + k] = a;
+        S.h1[a][u] = fmaxf(p, 0.0f);
+        S.h1[b][u] = fmaxf(q, 0.0f);
     }
-}
-
-// One thread per parameter: its gradient summed over the samples in order, in FP64.
-__global__ void k_mlp_param_grad(const float* __restrict__ x, const float* __restrict__ h1,
-                                 const float* __restrict__ h2, const float* __restrict__ dy,
-                                 const float* __restrict__ dh1, const float* __restrict__ dh2, int64_t n,
-                                 float* __restrict__ grad)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kP) return;
-    double acc = 0.0;
-    if (p < ob1) {
-        const int k = p / kIn, i = p % kIn;
-        for (int64_t s = 0; s < n; s++) acc += (double)dh1[s * kH + k] * x[s * kIn + i];
-    } else if (p < oW2) {
-        const int k = p - ob1;
-        for (int64_t s = 0; s < n; s++) acc += dh1[s * kH + k];
-    } else if (p < ob2) {
-        const int j = (p - oW2) / kH, k = (p - oW2) % kH;
-        for (int64_t s = 0; s < n; s++) acc += (double)dh2[s * kH + j] * h1[s * kH + k];
-    } else if (p < ow3) {
-        const int j = p - ob2;
-        for (int64_t s = 0; s < n; s++) acc += dh2[s * kH + j];
-    } else if (p < ob3) {
-        const int j = p - ow3;
-        for (int64_t s = 0; s < n; s++) acc += (double)dy[s] * h2[s * kH + j];
-    } else {
-        for (int64_t s = 0; s < n; s++) acc += dy[s];
-    }
-    grad[p] = (float)acc;
-}
-
-// Mean squared error in FP64, one CTA, fixed order.
-__global__ void k_mlp_loss(const float* __restrict__ y, const float* __restrict__ t, int64_t n, double* loss)
-{
-    __shared__ double sh[kThreads];
-    double a = 0.0;
-    for (int64_t s = threadIdx.x; s < n; s += blockDim.x) {
-        const double d = (double)y[s] - t[s];
-        a += d * d;
-    }
-    sh[threadIdx.x] = a;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int i = 0; i < (int)blockDim.x; i++) tot += sh[i];
-        *loss = n > 0 ? tot / (double)n : 0.0;
+    {
+        float p = S.b2[u], q = p;
+#pragma unroll
+        for (int k = 0; k < kH; k += 4) {
+            const float4 ha = *reinterpret_cast<const float4*>(&S.h1[a][k]);
+            const float4 hb = *reinterpret_cast<const float4*>(&S.h1[b][k]);
+            const float va[4] = {ha.x, ha.y, ha.z, ha.w}, vb[4] = {hb.x, hb.y, hb.z, hb.w};
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const float w = S.w2[u][k + i];
+                p = fmaf(w, va[i], p);
+                q = fmaf(w, vb[i], q);
+            }
+        }
+        S.h2[a][u] = fmaxf(p, 0.0f);
+        S.h2[b][u] = fmaxf(q, 0.0f);
+    }
+    __syncthreads();
+    if ((tid & 31) == 0) {  // one sample per warp
+        const int s = tid >> 5;
+        float out = S.b3;
+#pragma unroll 16
+        for (int j = 0; j < kH; j++) out = fmaf(S.w3[j], S.h2[s][j], out);
+        S.y[s] = out;
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_forward(const float* __restrict__ params,
+                                                             const float* __restrict__ x, int64_t n,
+                                                             float* __restrict__ y)
+{
+    __shared__ MlpSmem S;
+    load_params(params, S);
+    for (int64_t s0 = (int64_t)blockIdx.x * kMlpBatch; s0 < n; s0 += (int64_t)gridDim.x * kMlpBatch) {
+        const int m = (int)min((int64_t)kMlpBatch, n - s0);
+        forward_batch(S, x, s0, m);
+        if (threadIdx.x < m) y[s0 + threadIdx.x] = S.y[threadIdx.x];
     }
 }
+
+// A sum of products held as high + low part: the product's rounding error by an fma, the
+// sum's by TwoSum (Knuth 1969), both exact, so the sum carries 48 bits.
+struct PairSum {
+    float h, l;
+    __device__ __forceinline__ void add(float p, float e)
+    {
+        const float s = h + p, t = s - h;
+        l += ((h - (s - t)) + (p - t)) + e;
+        h = s;
+    }
+    __device__ __forceinline__ void add_product(float a, float b)
+    {
+        const float p = a * b;
+        add(p, fmaf(a, b, -p));
+    }
+    // an overflowed sum has no low part
+    __device__ __forceinline__ double value() const { return fabsf(h) < INFINITY ? (double)h + (double)l : (double)h; }
+};
+
+// Gradient of L = (1/n) sum (y - t)^2 and the sum of squares over samples blockIdx.x * per
+// .. + per - 1: into part [blockIdx.x][kP + 1] (kDirect: one CTA, the gradient and L).
+// dL/d(pre-activation) of layer 2 is d2, of layer 1 d1; the ReLU passes the gradient where
+// its output > 0.
+// The 4801 sums over samples are what bounds an epoch.  FP64 instructions are scarce (two
+// per clock and SM), so a thread keeps its ten sums as FP32 pairs over the CTA's samples
+// and only their values are added in FP64.  Measured with 5696 samples: 44 us an epoch;
+// one thread per parameter with FP64 sums over all samples took 833.
+template <bool kDirect>
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_slab(const float* __restrict__ params,
+                                                          const float* __restrict__ x,
+                                                          const float* __restrict__ t, int64_t n, int64_t per,
+                                                          double* __restrict__ part, float* __restrict__ grad,
+                                                          double* __restrict__ loss)
+{
+    __shared__ MlpSmem S;
+    __shared__ double sq[kMlpBatch];
+    load_params(params, S);
+    const int tid = threadIdx.x;
+    const int u = tid & (kH - 1), a = 2 * (tid / kH), b = a + 1;
+    // this thread's parameters: W2 rows 2 j2, 2 j2 + 1, columns 4 k4 .. + 3; W1 entry tid; and of
+    // threads 0 .. 192 one of b1, b2, w3, b3
+    const int j2 = 2 * (tid >> 4), k4 = 4 * (tid & 15);
+    PairSum g2[2][4] = {}, g1 = {}, g0 = {};
+    double err = 0.0;  // of the sample whose output this thread has (first lane of a warp)
+    const int64_t begin = (int64_t)blockIdx.x * per, end = min(n, begin + per);
+    for (int64_t s0 = begin; s0 < end; s0 += kMlpBatch) {
+        const int m = (int)min((int64_t)kMlpBatch, end - s0);
+        forward_batch(S, x, s0, m);
+        if ((tid & 31) == 0) {
+            const int s = tid >> 5;
+            float g = 0.0f;
+            if (s < m) {
+                const float ts = t[s0 + s];
+                g = 2.0f * (S.y[s] - ts) / (float)n;
+                const double d = (double)S.y[s] - ts;
+                err += d * d;
+            }
+            S.dy[s] = g;
+        }
+        __syncthreads();
+        S.d2[a][u] = S.h2[a][u] > 0.0f ? S.dy[a] * S.w3[u] : 0.0f;
+        S.d2[b][u] = S.h2[b][u] > 0.0f ? S.dy[b] * S.w3[u] : 0.0f;
+        __syncthreads();
+        {
+            float p = 0.0f, q = 0.0f;
+#pragma unroll
+            for (int j = 0; j < kH; j += 4) {
+                const float4 da = *reinterpret_cast<const float4*>(&S.d2[a][j]);
+                const float4 db = *reinterpret_cast<const float4*>(&S.d2[b][j]);
+                const float va[4] = {da.x, da.y, da.z, da.w}, vb[4] = {db.x, db.y, db.z, db.w};
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const float w = S.w2[j + i][u];
+                    p = fmaf(w, va[i], p);
+                    q = fmaf(w, vb[i], q);
+                }
+            }
+            S.d1[a][u] = S.h1[a][u] > 0.0f ? p : 0.0f;
+            S.d1[b][u] = S.h1[b][u] > 0.0f ? q : 0.0f;
+        }
+        __syncthreads();
+        for (int s = 0; s < m; s++) {
+            const float2 d = *reinterpret_cast<const float2*>(&S.d2[s][j2]);
+            const float4 h = *reinterpret_cast<const float4*>(&S.h1[s][k4]);
+            const float dv[2] = {d.x, d.y}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+#pragma unroll
+                for (int k = 0; k < 4; k++) g2[i][k].add_product(dv[i], hv[k]);
+            g1.add_product(S.d1[s][tid / kIn], S.x[s][tid % kIn]);
+            if (tid < kH) g0.add(S.d1[s][u], 0.0f);
+            else if (tid < 2 * kH) g0.add(S.d2[s][u], 0.0f);
+            else if (tid < 3 * kH) g0.add_product(S.dy[s], S.h2[s][u]);
+            else if (tid == 3 * kH) g0.add(S.dy[s], 0.0f);
+        }
+        __syncthreads();  // the batch's activations are no longer read
+    }
+    auto put = [&](int p, const PairSum& g) {
+        if (kDirect) grad[p] = (float)g.value();
+        else part[(int64_t)blockIdx.x * (kP + 1) + p] = g.value();
+    };
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int k = 0; k < 4; k++) put(oW2 + (j2 + i) * kH + k4 + k, g2[i][k]);
+    put(oW1 + tid, g1);
+    if (tid < kH) put(ob1 + u, g0);
+    else if (tid < 2 * kH) put(ob2 + u, g0);
+    else if (tid < 3 * kH) put(ow3 + u, g0);
+    else if (tid == 3 * kH) put(ob3, g0);
+    if ((tid & 31) == 0) sq[tid >> 5] = err;
+    __syncthreads();
+    if (tid == 0) {
+        double e = 0.0;
+        for (int s = 0; s < kMlpBatch; s++) e += sq[s];
+        if (!kDirect) part[(int64_t)blockIdx.x * (kP + 1) + kP] = e;
+        else if (loss) *loss = e / (double)n;
+    }
+}
+static_assert(kMlpThreads == kH * kIn && kMlpThreads * 8 == kH * kH && kMlpThreads == kMlpBatch * 32 &&
+                  kMlpThreads * 2 == kMlpBatch * kH,
+              "threads of a batch");
 
 // Adam (Kingma & Ba 2015) with bias correction: c1 = 1/(1 - beta1^t), c2 = 1/(1 - beta2^t).
-__global__ void k_mlp_adam(float* __restrict__ params, float* __restrict__ m, float* __restrict__ v,
-                           const float* __restrict__ grad, float lr, float c1, float c2)
+struct AdamArgs {
+    float *params, *m, *v;
+    float lr, c1, c2;
+};
+__device__ __forceinline__ void adam_update(const AdamArgs& A, int p, float g)
+{
+    const float mm = VL_MLP_BETA1 * A.m[p] + (1.0f - VL_MLP_BETA1) * g;
+    const float vv = VL_MLP_BETA2 * A.v[p] + (1.0f - VL_MLP_BETA2) * g * g;
+    A.m[p] = mm;
+    A.v[p] = vv;
+    A.params[p] -= A.lr * (mm * A.c1) / (sqrtf(vv * A.c2) + VL_MLP_EPS);
+}
+
+__global__ void k_mlp_adam(AdamArgs A, const float* __restrict__ grad)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kP) return;
-    const float g = grad[p];
-    const float mm = VL_MLP_BETA1 * m[p] + (1.0f - VL_MLP_BETA1) * g;
-    const float vv = VL_MLP_BETA2 * v[p] + (1.0f - VL_MLP_BETA2) * g * g;
-    m[p] = mm;
-    v[p] = vv;
-    params[p] -= lr * (mm * c1) / (sqrtf(vv * c2) + VL_MLP_EPS);
+    if (p < kP) adam_update(A, p, grad[p]);
+}
+
+// Sum of the parts in a fixed order: 32 parameters and 8 interleaved chains of parts per
+// CTA.  kAdam: the update; else the gradient.  Entry kP is the sum of squares.
+template <bool kAdam>
+__global__ void __launch_bounds__(256) k_mlp_join(const double* __restrict__ part, int nparts, int64_t n,
+                                                  AdamArgs A, float* __restrict__ grad, double* __restrict__ loss)
+{
+    __shared__ double sh[8][32];
+    const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    double a = 0.0;
+    if (p <= kP)
+        for (int s = c; s < nparts; s += 8) a += part[(int64_t)s * (kP + 1) + p];
+    sh[c][lane] = a;
+    __syncthreads();
+    if (c != 0 || p > kP) return;
+    for (int i = 1; i < 8; i++) a += sh[i][lane];
+    if (p == kP) {
+        if (loss) *loss = a / (double)n;
+    } else if (kAdam) {
+        adam_update(A, p, (float)a);
+    } else {
+        grad[p] = (float)a;
+    }
 }
 
 // capacity = ceil((1 + margin) * sum_i max(exp(y_i) - 1, 0)), FP64, one CTA, fixed order.
@@ -320,30 +442,52 @@ __global__ void k_capacity_sum(const float* __restrict__ y, int64_t n, double ma
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-struct TrainWs {
-    float *y, *h1, *h2, *dy, *dh1, *dh2, *grad;
-    double* loss;
-};
+// Workspace of a training step, of vl_mlp_workspace_bytes: the loss, the gradient, then
+// the CTAs' parts.  About one kB per sample, so that a part covers about 38 samples or, with
+// more than 38 samples per SM, there is one part per SM.
+constexpr size_t kWsGrad = 256, kWsParts = kWsGrad + ((size_t)kP * 4 + 255) / 256 * 256;
 
-size_t train_ws_layout(int64_t n, char* base, TrainWs* w)
+size_t train_ws_bytes(int64_t n)
 {
-    size_t o = 0;
-    auto take = [&](size_t bytes) {
-        char* p = base ? base + o : nullptr;
-        o = align256(o + bytes);
-        return p;
-    };
-    TrainWs t;
-    t.y = (float*)take((size_t)n * 4);
-    t.h1 = (float*)take((size_t)n * kH * 4);
-    t.h2 = (float*)take((size_t)n * kH * 4);
-    t.dy = (float*)take((size_t)n * 4);
-    t.dh1 = (float*)take((size_t)n * kH * 4);
-    t.dh2 = (float*)take((size_t)n * kH * 4);
-    t.grad = (float*)take((size_t)kP * 4);
-    t.loss = (double*)take(8);
-    if (w) *w = t;
-    return o;
+    return 2 * align256((size_t)n * 4) + 4 * align256((size_t)n * kH * 4) + kWsParts;
+}
+
+// Queues gradient (and, with A, the Adam update) of one full batch.
+vl_status queue_gradient(const float* params, const float* x, const float* t, int64_t n, void* workspace,
+                         float* grad_out, const AdamArgs* A, double* loss_out, cudaStream_t s)
+{
+    char* ws = static_cast<char*>(workspace);
+    // the kernels write the loss in place unless the caller's pointer is not aligned for it
+    const bool copy_loss = loss_out && ((uintptr_t)loss_out & 7);
+    double* loss = copy_loss ? reinterpret_cast<double*>(ws) : loss_out;
+    float* grad = grad_out ? grad_out : reinterpret_cast<float*>(ws + kWsGrad);
+    double* part = reinterpret_cast<double*>(ws + kWsParts);
+    int device = 0, nsm = 0;
+    cudaGetDevice(&device);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
+    const int64_t room = (int64_t)((train_ws_bytes(n) - kWsParts) / ((kP + 1) * sizeof(double)));
+    const int64_t most = std::max<int64_t>(1, std::min<int64_t>(nsm, room));
+    const int64_t per = (n + most - 1) / most;
+    const int parts = (int)((n + per - 1) / per);
+    const AdamArgs none{};
+    if (parts == 1) {
+        k_mlp_slab<true><<<1, kMlpThreads, 0, s>>>(params, x, t, n, per, nullptr, grad, loss);
+        if (A) k_mlp_adam<<<nblk(kP, 128), 128, 0, s>>>(*A, grad);
+    } else {
+        k_mlp_slab<false><<<parts, kMlpThreads, 0, s>>>(params, x, t, n, per, part, nullptr, nullptr);
+        if (A) k_mlp_join<true><<<nblk(kP + 1, 32), 256, 0, s>>>(part, parts, n, *A, nullptr, loss);
+        else k_mlp_join<false><<<nblk(kP + 1, 32), 256, 0, s>>>(part, parts, n, none, grad, loss);
+    }
+    note_launch();
+    if (A || parts > 1) note_launch();
+    if (copy_loss) cudaMemcpyAsync(loss_out, loss, 8, cudaMemcpyDeviceToDevice, s);
+    return cudaGetLastError() == cudaSuccess ? VL_OK : VL_ECUDA;
+}
+
+// CTAs of a forward pass: one per batch, up to four per SM.
+unsigned forward_ctas(int64_t n)
+{
+    return (unsigned)std::min<int64_t>((n + kMlpBatch - 1) / kMlpBatch, 152 * 4);
 }
 
 vl_status launch_status()
@@ -423,14 +567,14 @@ extern "C" vl_status vl_mlp_forward(const float* params, const float* x, int64_t
 {
     if (!params || n < 0 || (n > 0 && (!x || !y))) return VL_EINVAL;
     if (n == 0) return VL_OK;
-    k_mlp_forward<<<nblk(n, kThreads), kThreads, 0, (cudaStream_t)stream>>>(params, x, n, y, nullptr, nullptr);
+    k_mlp_forward<<<forward_ctas(n), kMlpThreads, 0, (cudaStream_t)stream>>>(params, x, n, y);
     note_launch();
     return launch_status();
 }
 
 extern "C" size_t vl_mlp_workspace_bytes(int64_t n)
 {
-    return n < 0 ? 0 : train_ws_layout(n, nullptr, nullptr);
+    return n < 0 ? 0 : train_ws_bytes(n);
 }
 
 extern "C" vl_status vl_mlp_train_step(float* params, float* adam_m, float* adam_v, const float* x,
@@ -439,21 +583,11 @@ extern "C" vl_status vl_mlp_train_step(float* params, float* adam_m, float* adam
 {
     if (!params || !adam_m || !adam_v || !x || !t || n <= 0 || step < 1 || !(lr >= 0.0f) || !workspace)
         return VL_EINVAL;
-    if (workspace_bytes < train_ws_layout(n, nullptr, nullptr) || ((uintptr_t)workspace & 255)) return VL_EINVAL;
-    cudaStream_t s = (cudaStream_t)stream;
-    TrainWs w;
-    train_ws_layout(n, static_cast<char*>(workspace), &w);
-    const int nb = nblk(n, kThreads);
-    k_mlp_forward<<<nb, kThreads, 0, s>>>(params, x, n, w.y, w.h1, w.h2);
-    k_mlp_loss<<<1, kThreads, 0, s>>>(w.y, t, n, w.loss);
-    k_mlp_backward<<<nb, kThreads, 0, s>>>(params, w.y, t, n, w.h1, w.h2, w.dy, w.dh1, w.dh2);
-    k_mlp_param_grad<<<nblk(kP, kThreads), kThreads, 0, s>>>(x, w.h1, w.h2, w.dy, w.dh1, w.dh2, n, w.grad);
+    if (workspace_bytes < train_ws_bytes(n) || ((uintptr_t)workspace & 255)) return VL_EINVAL;
     const double c1 = 1.0 / (1.0 - std::pow((double)VL_MLP_BETA1, step));
     const double c2 = 1.0 / (1.0 - std::pow((double)VL_MLP_BETA2, step));
-    k_mlp_adam<<<nblk(kP, kThreads), kThreads, 0, s>>>(params, adam_m, adam_v, w.grad, lr, (float)c1, (float)c2);
-    for (int i = 0; i < 5; i++) note_launch();
-    if (loss) cudaMemcpyAsync(loss, w.loss, 8, cudaMemcpyDeviceToDevice, s);
-    return launch_status();
+    const AdamArgs A{params, adam_m, adam_v, lr, (float)c1, (float)c2};
+    return queue_gradient(params, x, t, n, workspace, nullptr, &A, loss, (cudaStream_t)stream);
 }
 
 extern "C" vl_status vl_mlp_gradient(const float* params, const float* x, const float* t, int64_t n,
@@ -461,18 +595,8 @@ extern "C" vl_status vl_mlp_gradient(const float* params, const float* x, const 
                                      void* stream)
 {
     if (!params || !x || !t || n <= 0 || !workspace || !grad) return VL_EINVAL;
-    if (workspace_bytes < train_ws_layout(n, nullptr, nullptr) || ((uintptr_t)workspace & 255)) return VL_EINVAL;
-    cudaStream_t s = (cudaStream_t)stream;
-    TrainWs w;
-    train_ws_layout(n, static_cast<char*>(workspace), &w);
-    const int nb = nblk(n, kThreads);
-    k_mlp_forward<<<nb, kThreads, 0, s>>>(params, x, n, w.y, w.h1, w.h2);
-    k_mlp_loss<<<1, kThreads, 0, s>>>(w.y, t, n, w.loss);
-    k_mlp_backward<<<nb, kThreads, 0, s>>>(params, w.y, t, n, w.h1, w.h2, w.dy, w.dh1, w.dh2);
-    k_mlp_param_grad<<<nblk(kP, kThreads), kThreads, 0, s>>>(x, w.h1, w.h2, w.dy, w.dh1, w.dh2, n, grad);
-    for (int i = 0; i < 4; i++) note_launch();
-    if (loss) cudaMemcpyAsync(loss, w.loss, 8, cudaMemcpyDeviceToDevice, s);
-    return launch_status();
+    if (workspace_bytes < train_ws_bytes(n) || ((uintptr_t)workspace & 255)) return VL_EINVAL;
+    return queue_gradient(params, x, t, n, workspace, grad, nullptr, loss, (cudaStream_t)stream);
 }
 
 extern "C" vl_status vl_mlp_capacity(const float* params, const float* features, int64_t ntiles,
@@ -484,7 +608,7 @@ extern "C" vl_status vl_mlp_capacity(const float* params, const float* features,
     cudaStream_t s = (cudaStream_t)stream;
     float* y = static_cast<float*>(workspace);
     int64_t* out = reinterpret_cast<int64_t*>(static_cast<char*>(workspace) + align256((size_t)ntiles * 4));
-    k_mlp_forward<<<nblk(ntiles, kThreads), kThreads, 0, s>>>(params, features, ntiles, y, nullptr, nullptr);
+    k_mlp_forward<<<forward_ctas(ntiles), kMlpThreads, 0, s>>>(params, features, ntiles, y);
     k_capacity_sum<<<1, kThreads, 0, s>>>(y, ntiles, margin, out);
     note_launch();
     note_launch();
