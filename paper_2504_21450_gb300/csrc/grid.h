@@ -134,6 +134,22 @@ vl_status moments(Grid* g, double* out, int on_device);
 // released by the caller once the stream has passed.
 vl_status queue_cell_moments(Grid* g, double* d_out, void** scratch);
 vl_status tile_features(Grid* g, int edge, float* feat, float* uni);
+// ---- lists.cu --------------------------------------------------------------
+struct Window;  // blocks.cuh
+// Parts that the block ids of a window's lists are split into.
+int list_parts(const Grid* g, const Window& W);
+// cnt[part][window cell] = blocks of the cell in earlier parts (not written with one part);
+// total (optional) per cell.
+void launch_list_counts(Grid* g, const uint64_t* kbits, const Window& W, uint32_t* cnt, uint32_t* total);
+// Ids and values of the window's blocks (kbits) to lists at `off` / values of such lists to
+// the blocks' slots; start from launch_list_counts; host: vals is a mapped host buffer.
+void launch_blocks_out(Grid* g, const Layout& L, const Window& W, const int64_t* off, const uint32_t* start,
+                       uint16_t* ids, float* vals, bool host);
+void launch_blocks_in(Grid* g, const Layout& L, const Window& W, const int64_t* off, const uint32_t* start,
+                      const float* vals);
+// Marks the listed blocks of every cell in ubits; err |= 2 (id out of range), 4 (ids not
+// strictly increasing within a cell).
+void launch_mark_cells(Grid* g, const int64_t* off, const uint16_t* ids, int64_t M, uint64_t* ubits, int* err);
 // ---- moments.cu ------------------------------------------------------------
 // The velocity mesh is narrow enough for queue_moments, which is queue_cell_moments for
 // such meshes.

@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "blocks.cuh"
 #include "grid.h"
 
 namespace vlgt {
@@ -341,81 +342,13 @@ __global__ void k_scatter(GridGeom G, LayoutView L, const uint16_t* __restrict__
     static_cast<typename Codec<kCodec>::T*>(L.pool)[dst] = Codec<kCodec>::enc(f, inv);
 }
 
-// ---- layout -> per-cell lists ----------------------------------------------------
-struct Window {
-    int o[3], s[3];
-    int64_t ncell;
-};
-
-// global (x, row) of window cell wc (x fastest), wrapping periodically
-__device__ __forceinline__ void window_cell(const GridGeom& G, const Window& Wn, int64_t wc, int& x,
-                                            int64_t& row)
-{
-    int wx = (int)(wc % Wn.s[0]);
-    int64_t r = wc / Wn.s[0];
-    int wy = (int)(r % Wn.s[1]);
-    int wz = (int)(r / Wn.s[1]);
-    x = wrapi(Wn.o[0] + wx, G.n[0]);
-    int y = wrapi(Wn.o[1] + wy, G.n[1]);
-    int z = wrapi(Wn.o[2] + wz, G.n[2]);
-    row = y + (int64_t)G.n[1] * z;
-}
-
-__global__ void k_cell_counts(GridGeom G, Window Wn, const uint64_t* __restrict__ kbits,
-                              uint32_t* __restrict__ cnt)
-{
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= Wn.ncell) return;
-    int x;
-    int64_t row;
-    window_cell(G, Wn, c, x, row);
-    int64_t wo = row * G.W + (x >> 6);
-    uint64_t bit = 1ull << (x & 63);
-    uint32_t k = 0;
-    for (int b = 0; b < G.nb; b++) k += (kbits[(int64_t)b * G.RW + wo] & bit) ? 1u : 0u;
-    cnt[c] = k;
-}
-
+// ---- layout -> per-cell lists (values: lists.cu) --------------------------------------
 __global__ void k_offsets64(const uint32_t* __restrict__ excl, const int64_t* __restrict__ chunk_base,
                             int64_t chunk, int64_t N, int64_t* __restrict__ off)
 {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c < N) off[c] = chunk_base[c / chunk] + excl[c];
     if (c == 0) off[N] = chunk_base[(N + chunk - 1) / chunk];
-}
-
-__global__ void k_fill_ids(GridGeom G, Window Wn, LayoutView L, const int64_t* __restrict__ off,
-                           uint16_t* __restrict__ ids, int64_t* __restrict__ rank_of)
-{
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= Wn.ncell) return;
-    int x;
-    int64_t row;
-    window_cell(G, Wn, c, x, row);
-    int64_t wo = row * G.W + (x >> 6);
-    uint64_t bit = 1ull << (x & 63);
-    int64_t o = off[c];
-    for (int b = 0; b < G.nb; b++) {
-        if (L.kbits[(int64_t)b * G.RW + wo] & bit) {
-            ids[o] = (uint16_t)b;
-            rank_of[o] = cell_rank(L, G, b, x, row, false);
-            o++;
-        }
-    }
-}
-
-template <int kCodec>
-__global__ void k_gather(LayoutView L, const uint16_t* __restrict__ ids,
-                         const int64_t* __restrict__ rank_of, float* __restrict__ vals, int64_t M)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M * 64) return;
-    int64_t t = i >> 6;
-    int v = (int)(i & 63);
-    int b = ids[t];
-    const auto* pool = static_cast<const typename Codec<kCodec>::T*>(L.pool);
-    const int64_t e = ((int64_t)L.base[b] * 4 + (int64_t)(v >> 4) * L.cnt[b] + rank_of[t]) * kChunk + (v & 15);
-    vals[i] = Codec<kCodec>::dec(pool[e], kCodec ? L.scale[e >> 4] : 1.0f);
 }
 
 // ---- moments -----------------------------------------------------------------------
@@ -701,6 +634,20 @@ static void* mapped_host(const void* p)
     return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+namespace {
+Window make_window(const GridGeom& G, const int* origin, const int* size)
+{
+    Window Wn;
+    Wn.ncell = 1;
+    for (int d = 0; d < 3; d++) {
+        Wn.o[d] = origin ? origin[d] : 0;
+        Wn.s[d] = size ? size[d] : G.n[d];
+        Wn.ncell *= Wn.s[d];
+    }
+    return Wn;
+}
+}  // namespace
+
 vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* ids_in,
                      const float* vals_in, int on_device)
 {
@@ -726,13 +673,23 @@ vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* 
     }
     Layout& L = g->lay[g->cur];
     size_t words = (size_t)G.nb * (size_t)G.RW;
-    int64_t* cell_of = (int64_t*)sc.get((size_t)std::max<int64_t>(M, 1) * 8);
+    // values that the device can read in place go to their slots cell by cell (lists.cu); a
+    // list that is copied in chunks of blocks goes value by value, each block's cell looked up
+    const bool direct = on_device || mapped;
+    const Window all = make_window(G, nullptr, nullptr);
+    int64_t* cell_of = direct ? nullptr : (int64_t*)sc.get((size_t)std::max<int64_t>(M, 1) * 8);
+    uint32_t* start = direct ? (uint32_t*)sc.get((size_t)list_parts(g, all) * G.N * 4) : nullptr;
     int* err = (int*)sc.get(sizeof(int));
-    if (!cell_of || !err) return fail(g, VL_ENOMEM, "vl_set_blocks: scratch allocation failed");
+    if ((!cell_of && !start) || !err) return fail(g, VL_ENOMEM, "vl_set_blocks: scratch allocation failed");
     cudaMemsetAsync(err, 0, sizeof(int), s);
     cudaMemsetAsync(L.ubits, 0, words * 8, s);
     k_check_offsets<<<nblk(G.N + 1, 256), 256, 0, s>>>(off, G.N, M, err); note_launch();
-    if (M > 0) { k_mark<<<nblk(M, 256), 256, 0, s>>>(G, off, ids, M, L.ubits, cell_of, err); note_launch(); }
+    if (M > 0 && direct) {
+        launch_mark_cells(g, off, ids, M, L.ubits, err);
+    } else if (M > 0) {
+        k_mark<<<nblk(M, 256), 256, 0, s>>>(G, off, ids, M, L.ubits, cell_of, err);
+        note_launch();
+    }
     cudaMemcpyAsync(g->host_scalar, err, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(g, e, "vl_set_blocks");
@@ -756,7 +713,6 @@ vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* 
     float* stage_buf[2] = {nullptr, nullptr};
     cudaEvent_t ready = nullptr, copied[2] = {nullptr, nullptr}, used[2] = {nullptr, nullptr};
     const bool staged = M > 0 && !on_device && !mapped;
-    const bool direct = on_device || mapped;  // the kernels read vals in place
     // two buffers when more than one chunk goes through them
     const int nbuf = ((M + chunk - 1) / chunk > 1) ? 2 : 1;
     if (staged) {
@@ -777,11 +733,15 @@ vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* 
         cudaStreamWaitEvent(g->copy_stream, ready, 0);
     }
     int64_t k = 0;  // chunk counter (staging buffer k % nbuf)
-    for (int64_t t0 = 0; t0 < M; t0 += (direct ? M : chunk), k++) {
-        const int64_t m = direct ? M : std::min(chunk, M - t0);
+    if (direct && M > 0) {
+        launch_list_counts(g, L.kbits, all, start, nullptr);
+        launch_blocks_in(g, L, all, off, start, vals);
+    }
+    for (int64_t t0 = 0; staged && t0 < M; t0 += chunk, k++) {
+        const int64_t m = std::min(chunk, M - t0);
         const int bi = (int)(k % nbuf);
-        const float* v = direct ? vals : stage_buf[bi];
-        if (staged) {
+        const float* v = stage_buf[bi];
+        {
             if (k >= nbuf) cudaStreamWaitEvent(g->copy_stream, used[bi], 0);  // chunk k-nbuf consumed
             cudaMemcpyAsync(stage_buf[bi], vals_in + t0 * 64, (size_t)m * 256, cudaMemcpyHostToDevice,
                             g->copy_stream);
@@ -792,7 +752,7 @@ vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* 
             k_scatter<decltype(c)::value><<<nblk(m * 64, 256), 256, 0, s>>>(G, L.view(), ids, cell_of, v, t0, m);
         });
         note_launch();
-        if (staged) cudaEventRecord(used[bi], s);
+        cudaEventRecord(used[bi], s);
     }
     if (staged) {
         cudaStreamSynchronize(s);  // every copy was waited for by a kernel on s
@@ -807,20 +767,6 @@ vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* 
     g->has_state = true;
     return VL_OK;
 }
-
-namespace {
-Window make_window(const GridGeom& G, const int* origin, const int* size)
-{
-    Window Wn;
-    Wn.ncell = 1;
-    for (int d = 0; d < 3; d++) {
-        Wn.o[d] = origin ? origin[d] : 0;
-        Wn.s[d] = size ? size[d] : G.n[d];
-        Wn.ncell *= Wn.s[d];
-    }
-    return Wn;
-}
-}  // namespace
 
 // Per-cell lists of a box window of the grid (the whole grid when origin/size are
 // NULL).  With count_only, only *count is produced.
@@ -843,9 +789,11 @@ vl_status get_window(Grid* g, const int* origin, const int* size, int64_t capaci
     uint32_t* cexc = (uint32_t*)sc.get((size_t)nchunk * chunk * 4);
     uint32_t* ctot = (uint32_t*)sc.get((size_t)nchunk * 4);
     int64_t* cbase = (int64_t*)sc.get(((size_t)nchunk + 1) * 8);
-    if (!ccnt || !cexc || !ctot || !cbase) return fail(g, VL_ENOMEM, "block listing: scratch allocation failed");
+    uint32_t* start = (uint32_t*)sc.get((size_t)list_parts(g, Wn) * Wn.ncell * 4);
+    if (!ccnt || !cexc || !ctot || !cbase || !start)
+        return fail(g, VL_ENOMEM, "block listing: scratch allocation failed");
     cudaMemsetAsync(ccnt, 0, (size_t)nchunk * chunk * 4, s);
-    k_cell_counts<<<nblk(Wn.ncell, 256), 256, 0, s>>>(G, Wn, L.kbits, ccnt); note_launch();
+    launch_list_counts(g, L.kbits, Wn, start, ccnt);
     launch_seg_scan(ccnt, cexc, ctot, chunk, nchunk, s, nullptr);
     launch_base_scan(ctot, cbase, nchunk, s, nullptr);
     cudaMemcpyAsync(g->host_scalar, cbase + nchunk, 8, cudaMemcpyDeviceToHost, s);
@@ -858,21 +806,14 @@ vl_status get_window(Grid* g, const int* origin, const int* size, int64_t capaci
         return fail(g, VL_ECAPACITY, "vl_get_blocks: capacity " + std::to_string(capacity) +
                                          " < " + std::to_string(M) + " blocks");
     if (M > 0 && (!ids_out || !vals_out)) return fail(g, VL_EINVAL, "vl_get_blocks: null pointer");
-    int64_t* rank_of = (int64_t*)sc.get((size_t)std::max<int64_t>(M, 1) * 8);
     int64_t* d_off = on_device ? off_out : (int64_t*)sc.get((size_t)(Wn.ncell + 1) * 8);
     uint16_t* d_ids = on_device ? ids_out : (uint16_t*)sc.get((size_t)std::max<int64_t>(M, 1) * 2);
-    // values into a page-locked host buffer: the gather kernel writes them in place
+    // values into a page-locked host buffer: the kernel writes them in place
     float* mapped = (!on_device && M > 0) ? static_cast<float*>(mapped_host(vals_out)) : nullptr;
     float* d_vals = on_device ? vals_out : (mapped ? mapped : (float*)sc.get((size_t)std::max<int64_t>(M, 1) * 256));
-    if (!rank_of || !d_off || !d_ids || !d_vals) return fail(g, VL_ENOMEM, "vl_get_blocks: scratch allocation failed");
+    if (!d_off || !d_ids || !d_vals) return fail(g, VL_ENOMEM, "vl_get_blocks: scratch allocation failed");
     k_offsets64<<<nblk(Wn.ncell + 1, 256), 256, 0, s>>>(cexc, cbase, chunk, Wn.ncell, d_off); note_launch();
-    k_fill_ids<<<nblk(Wn.ncell, 128), 128, 0, s>>>(G, Wn, L.view(), d_off, d_ids, rank_of); note_launch();
-    if (M > 0) {
-        with_codec(g->codec, [&](auto c) {
-            k_gather<decltype(c)::value><<<nblk(M * 64, 256), 256, 0, s>>>(L.view(), d_ids, rank_of, d_vals, M);
-        });
-        note_launch();
-    }
+    if (M > 0) launch_blocks_out(g, L, Wn, d_off, start, d_ids, d_vals, mapped != nullptr);
     if (!on_device) {
         cudaMemcpyAsync(off_out, d_off, (size_t)(Wn.ncell + 1) * 8, cudaMemcpyDeviceToHost, s);
         if (M > 0) {
@@ -899,7 +840,8 @@ vl_status get_blocks(Grid* g, int64_t capacity, int64_t* off_out, uint16_t* ids_
 
 namespace {
 // Window block t -> its cell in the grid (planes from z0, wrapping); err |= 1 when the
-// cell does not hold that block id in the current layout, 2 when the id is out of range.
+// cell does not hold that block id in the current layout, 2 when the id is out of range, 4
+// when the ids of a cell do not increase.
 __global__ void k_window_cells(GridGeom G, LayoutView L, const int64_t* __restrict__ off_w, int64_t nw,
                                const uint16_t* __restrict__ ids_w, int64_t Mw, int z0,
                                int64_t* __restrict__ cell_of, int* err)
@@ -915,6 +857,7 @@ __global__ void k_window_cells(GridGeom G, LayoutView L, const int64_t* __restri
         return;
     }
     cell_of[t] = c;
+    if (t > 0 && t > off_w[wc] && ids_w[t - 1] >= b) atomicOr(err, 4);
     const int x = (int)(c % G.n[0]);
     const int64_t wi = (int64_t)b * G.RW + (c / G.n[0]) * G.W + (x >> 6);
     if (!((L.kbits[wi] >> (x & 63)) & 1ull)) atomicOr(err, 1);
@@ -974,21 +917,31 @@ vl_status set_blocks_planes(Grid* g, int z0, int nplanes, int64_t Mw, const int6
         if (st0 != VL_OK) return st0;
         if (Mcur == Mw) {
             int64_t* cell_of = (int64_t*)sc.get((size_t)std::max<int64_t>(Mw, 1) * 8);
-            int* err = (int*)sc.get(sizeof(int));
+            int* err = (int*)sc.get(2 * sizeof(int));  // of the blocks, of the offsets
             if (!cell_of || !err) return fail(g, VL_ENOMEM, "vl_set_blocks_planes: scratch allocation failed");
             Layout& L = g->lay[g->cur];
-            cudaMemsetAsync(err, 0, sizeof(int), s);
+            cudaMemsetAsync(err, 0, 2 * sizeof(int), s);
+            k_check_offsets<<<nblk(nw + 1, 256), 256, 0, s>>>(off_w, nw, Mw, err + 1);
+            note_launch();
             if (Mw > 0) {
                 k_window_cells<<<nblk(Mw, 256), 256, 0, s>>>(G, L.view(), off_w, nw, ids_w, Mw, z0, cell_of, err);
                 note_launch();
             }
-            cudaMemcpyAsync(g->host_scalar, err, sizeof(int), cudaMemcpyDeviceToHost, s);
+            cudaMemcpyAsync(g->host_scalar, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s);
             cudaError_t e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return cuda_fail(g, e, "vl_set_blocks_planes");
             const int herr = (int)(g->host_scalar[0] & 0xffffffff);
+            const bool sorted = (herr & 4) == 0 && (g->host_scalar[0] >> 32) == 0;
             if (herr & 2) return fail(g, VL_EINVAL, "vl_set_blocks_planes: block id out of range of the velocity mesh");
-            if (herr == 0) {
-                if (Mw > 0) {
+            if ((herr & 1) == 0) {
+                if (Mw > 0 && sorted) {
+                    // the lists are the window's blocks, cell by cell
+                    const Window W = make_window(G, origin, size);
+                    uint32_t* start = (uint32_t*)sc.get((size_t)list_parts(g, W) * nw * 4);
+                    if (!start) return fail(g, VL_ENOMEM, "vl_set_blocks_planes: scratch allocation failed");
+                    launch_list_counts(g, L.kbits, W, start, nullptr);
+                    launch_blocks_in(g, L, W, off_w, start, vals_w);
+                } else if (Mw > 0) {
                     with_codec(g->codec, [&](auto c) {
                         k_scatter<decltype(c)::value>
                             <<<nblk(Mw * 64, 256), 256, 0, s>>>(G, L.view(), ids_w, cell_of, vals_w, 0, Mw);

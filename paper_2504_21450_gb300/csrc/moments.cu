@@ -10,10 +10,7 @@
 // over single values would give them: one pass over f instead of two, 0.4 FP64
 // instructions per value instead of 28.
 //
-// A warp takes eight cells that are neighbours along x, four lanes each: a lane loads the
-// 16 bytes of one vx row, so a load instruction covers eight 64-byte chunks in a row.  The
-// warp walks the block ids in order, 32 bitmap words at a time, with the next block's
-// values in flight while one is summed.
+// A warp takes eight cells (blocks.cuh).
 //
 // Measured (64x32x16 cells x 32^3 velocity cells, 4.3 GB of f, 0.63 ms at the copy rate):
 // 1.16 ms per call, total mass 0.69; the kernel for any mesh, which sums every value
@@ -24,13 +21,13 @@
 #include <algorithm>
 #include <cmath>
 
+#include "blocks.cuh"
 #include "grid.h"
 
 namespace vlgt {
 
 namespace {
 
-constexpr int kGroup = 8;        // cells of a warp
 constexpr int kMaxRun = 8;       // blocks summed in FP32 pairs before the sum goes to FP64
 constexpr int kWarps = 8;        // warps of a CTA, at most
 
@@ -73,106 +70,12 @@ __device__ __forceinline__ Pair transpose_sum(const Pair (&p)[4], int k)
     return add(odd ? a1 : a0, shfl_xor(odd ? a0 : a1, 1));
 }
 
-// One vx row of each of a block's four chunks, as stored.
-template <int kCodec>
-struct Rows {
-    float4 v[4];
-    __device__ __forceinline__ void load(const LayoutView& L, int64_t chunk, uint32_t cnt, int k, bool has)
-    {
-#pragma unroll
-        for (int q = 0; q < 4; q++)
-            v[q] = has ? __ldcs(reinterpret_cast<const float4*>(static_cast<const float*>(L.pool) +
-                                                                 (chunk + (int64_t)q * cnt) * kChunk) + k)
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __device__ __forceinline__ float4 get(int q) const { return v[q]; }
-};
-template <int kCodec>
-struct Codes {
-    uint2 v[4];
-    float s[4];
-    __device__ __forceinline__ void load(const LayoutView& L, int64_t chunk, uint32_t cnt, int k, bool has)
-    {
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int64_t c = chunk + (int64_t)q * cnt;
-            v[q] = has ? __ldcs(reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(L.pool) + c * kChunk) + k)
-                       : make_uint2(0u, 0u);
-            s[q] = has ? L.scale[c] : 0.0f;
-        }
-    }
-    __device__ __forceinline__ float4 get(int q) const
-    {
-        using T = typename Codec<kCodec>::T;
-        const T* h = reinterpret_cast<const T*>(&v[q]);
-        return make_float4(Codec<kCodec>::dec(h[0], s[q]), Codec<kCodec>::dec(h[1], s[q]),
-                           Codec<kCodec>::dec(h[2], s[q]), Codec<kCodec>::dec(h[3], s[q]));
-    }
-};
-template <> struct Rows<1> : Codes<1> {};
-template <> struct Rows<2> : Codes<2> {};
-
 // Groups of eight cells along x, row by row.
 struct Groups {
     int per_row;     // groups of a row
     int64_t total;   // groups
-    int split;       // the block ids are split over this many CTAs (small grids)
-    int ids;         // block ids of a part (a multiple of 32)
+    int split, ids;  // parts of the block ids, ids of a part
 };
-
-// The block ids of one part that group g holds, in ascending order: body(id, rows, has)
-// with this lane's rows of the block.
-template <int kCodec, class Body>
-__device__ __forceinline__ void for_blocks(const GridGeom& G, const LayoutView& L, const Groups& P, int64_t grp,
-                                           int b_begin, int b_end, Body&& body)
-{
-    const int lane = threadIdx.x & 31, j = lane >> 2, k = lane & 3;
-    const int64_t row = grp / P.per_row;
-    const int x0 = (int)(grp - row * P.per_row) * kGroup;
-    const int64_t word = row * G.W + (x0 >> 6);  // the eight cells share one bitmap word
-    const int sh = x0 & 63;
-    auto kept = [&](int b) -> uint64_t { return b < b_end ? L.kbits[(int64_t)b * G.RW + word] : 0ull; };
-    uint64_t kw = kept(b_begin + lane);
-    for (int b0 = b_begin; b0 < b_end; b0 += 32) {
-        const unsigned k8 = (unsigned)(kw >> sh) & 0xffu;
-        unsigned m = __ballot_sync(0xffffffffu, k8 != 0u);
-        kw = kept(b0 + 32 + lane);  // the next words, while this batch is summed
-        if (!m) continue;
-        // lane i: cells (kept, slots), first chunk and chunk stride of block id b0 + i
-        unsigned bits = 0u;
-        int64_t first = 0;
-        uint32_t cnt = 0u;
-        if (k8) {
-            const int b = b0 + lane;
-            const uint64_t u = L.ubits[(int64_t)b * G.RW + word];
-            bits = k8 | ((unsigned)(u >> sh) & 0xffu) << 8;
-            first = L.base[b] * 4 + L.woff[(int64_t)b * G.RW + word] + __popcll(u & ((1ull << sh) - 1ull));
-            cnt = L.cnt[b];
-        }
-        Rows<kCodec> cur, nxt;
-        bool has = false, has_nxt = false;
-        auto fetch = [&](int i, Rows<kCodec>& r) -> bool {
-            const unsigned bi = __shfl_sync(0xffffffffu, bits, i);
-            const int64_t f = __shfl_sync(0xffffffffu, first, i);
-            const uint32_t c = __shfl_sync(0xffffffffu, cnt, i);
-            const bool h = (bi >> j) & 1u;
-            r.load(L, f + __popc((bi >> 8) & ((1u << j) - 1u)), c, k, h);
-            return h;
-        };
-        int i = __ffs(m) - 1;
-        has = fetch(i, cur);
-        while (true) {
-            m &= m - 1u;
-            const int in = m ? __ffs(m) - 1 : -1;
-            if (in >= 0) has_nxt = fetch(in, nxt);
-            body(b0 + i, cur, has);
-            if (in < 0) break;
-            i = in;
-            cur = nxt;
-            has = has_nxt;
-        }
-    }
-}
 
 // n V_d and P_dd of the group's cells from their marginals acc[(first index of d + i) *
 // kGroup + cell].
@@ -238,7 +141,14 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_marginals(GridGeom G, Layout
         run = 0;
     };
     const int b_begin = blockIdx.y * P.ids, b_end = min(G.nb, b_begin + P.ids);
-    for_blocks<kCodec>(G, L, P, grp, b_begin, b_end, [&](int b, const Rows<kCodec>& r, bool) {
+    const int64_t row = grp / P.per_row;
+    const int x0 = (int)(grp - row * P.per_row) * kGroup;
+    auto load = [&](int, bool has, int64_t chunk, uint32_t cnt) {
+        Rows<kCodec> r;
+        r.load(L, chunk, cnt, k, has);
+        return r;
+    };
+    for_blocks<Rows<kCodec>>(G, L, row, x0, 0xffu, b_begin, b_end, load, [&](int b, const Rows<kCodec>& r, bool, int64_t, uint32_t) {
         const int brow = b / G.nbx, bx = b - brow * G.nbx;
         if (brow != row_of_run || run == kMaxRun) {
             flush();
@@ -327,7 +237,14 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_density(GridGeom G, LayoutVi
     Pair p{0.f, 0.f};
     int run = 0;
     const int b_begin = blockIdx.y * P.ids, b_end = min(G.nb, b_begin + P.ids);
-    for_blocks<kCodec>(G, L, P, grp, b_begin, b_end, [&](int, const Rows<kCodec>& r, bool) {
+    const int64_t row = grp / P.per_row;
+    const int x0 = (int)(grp - row * P.per_row) * kGroup;
+    auto load = [&](int, bool has, int64_t chunk, uint32_t cnt) {
+        Rows<kCodec> r;
+        r.load(L, chunk, cnt, k, has);
+        return r;
+    };
+    for_blocks<Rows<kCodec>>(G, L, row, x0, 0xffu, b_begin, b_end, load, [&](int, const Rows<kCodec>& r, bool, int64_t, uint32_t) {
         Pair s{0.f, 0.f};
 #pragma unroll
         for (int q = 0; q < 4; q++) {
@@ -353,8 +270,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_density(GridGeom G, LayoutVi
     sum += value(p);
     sum += __shfl_xor_sync(0xffffffffu, sum, 1);
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-    const int64_t row = grp / P.per_row;
-    const int x = (int)(grp - row * P.per_row) * kGroup + j;
+    const int x = x0 + j;
     if (k == 0 && x < G.n[0]) dens[(int64_t)blockIdx.y * G.N + row * G.n[0] + x] = sum * (V.dv[0] * V.dv[1] * V.dv[2]);
 }
 
@@ -379,20 +295,15 @@ VMesh vmesh_of(const Grid* g)
     return V;
 }
 
-// Enough warps for the chip: small grids split the block ids, in parts of at least 64 (two
-// rounds of bitmap words); a group's ids are a serial chain.  16 warps per SM already hide
-// the loads.
 Groups groups_of(const Grid* g, int nsm)
 {
     const GridGeom& G = g->geom;
     Groups P;
     P.per_row = (G.n[0] + kGroup - 1) / kGroup;
     P.total = (int64_t)P.per_row * G.R;
-    const int64_t want = (int64_t)nsm * 16;
-    const int64_t most = std::max(1, (G.nb + 63) / 64);
-    const int64_t split = std::max<int64_t>(1, std::min(most, want / std::max<int64_t>(P.total, 1)));
-    P.ids = (int)(((G.nb + split - 1) / split + 31) / 32 * 32);
-    P.split = (G.nb + P.ids - 1) / P.ids;
+    const Parts s = parts_of(G.nb, P.total, (int64_t)nsm * 16, 64);  // a part has marginals to join
+    P.split = s.split;
+    P.ids = s.ids;
     return P;
 }
 
