@@ -41,6 +41,7 @@ struct PassArgs {
     uint8_t* keepq;
     StepCounters* ctr;
     int64_t groups;     // pencil groups per block id
+    int lg_pen;         // vector kernel: an item has 2^lg_pen pencils (kPen4 times a power of two)
     // vector kernel, list mode: work list of the (block id, pencil group) pairs that hold
     // any slot of the next layout (items[0 .. item_base[nb]) = b * groups + group), taken
     // by a persistent grid through the counter `next`
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(kThreads3) k_pass(PassArgs P)
 constexpr int kPen4 = 16;
 constexpr int kThreads4 = kPen4 * 16;
 constexpr int kBatch4 = 8;
+constexpr int kItemCells = 512;  // FP32: cells of an item's pencils end to end, at most (or one pencil)
 
 template <int kCodec>
 __device__ __forceinline__ void load4(const typename Codec<kCodec>::T* p, float sc, float (&o)[4])
@@ -291,9 +293,9 @@ __device__ bool row_has(const uint64_t* rowp, int xlo, int xhi)
     return acc != 0;
 }
 
-// flags[b][grp] = 1 when a pencil of group grp (pencils kPen4 grp .. kPen4 grp + kPen4 - 1
-// along dim, in pencil_cell's numbering) holds a slot of block id b in the layout
-__global__ void k_pass_groups(GridGeom G, const uint64_t* __restrict__ ubits, int dim, int64_t ngroups,
+// flags[b][grp] = 1 when a pencil of group grp (pen pencils along dim from pen * grp on, in
+// pencil_cell's numbering) holds a slot of block id b in the layout
+__global__ void k_pass_groups(GridGeom G, const uint64_t* __restrict__ ubits, int dim, int pen, int64_t ngroups,
                               uint32_t* __restrict__ flags)
 {
     if (aborted(G.abort)) return;
@@ -304,14 +306,14 @@ __global__ void k_pass_groups(GridGeom G, const uint64_t* __restrict__ ubits, in
     const uint64_t* seg = ubits + (int64_t)b * G.RW;
     const int nd = G.n[dim];
     const int64_t npen = G.N / nd;
-    const int64_t p0 = grp * kPen4, p1 = min(p0 + kPen4, npen);
+    const int64_t p0 = grp * pen, p1 = min(p0 + pen, npen);
     bool any = false;
     if (dim == 0) {
         // pencils are rows
         for (int64_t row = p0; row < p1 && !any; row++)
             for (int w = 0; w < G.W && !any; w++) any = seg[row * G.W + w] != 0;
     } else {
-        // pencil p = x + nx o (o = z along y, y along z): the group is at most two runs of x
+        // pencil p = x + nx o (o = z along y, y along z): runs of x
         const int nx = G.n[0];
         for (int64_t p = p0; p < p1 && !any;) {
             const int64_t o = p / nx;
@@ -328,7 +330,8 @@ __global__ void k_pass_groups(GridGeom G, const uint64_t* __restrict__ ubits, in
 }
 
 // kLast: the last pass (keep flags and mass, which need the values the state now holds).
-// An item is one (block id, group of kPen4 pencils) pair.  kList: a persistent grid takes
+// An item is one (block id, group of pencils) pair: kPen4 pencils, or several times as many
+// where pencils are short (run_3pass), swept kPen4 at a time.  kList: a persistent grid takes
 // the pairs of the work list and skips batches of positions with no slot; otherwise one
 // CTA per pair (a fully dense layout, where every pair is an item).
 template <bool kLim, int kCodec, bool kLast, bool kList>
@@ -336,10 +339,10 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
 {
     using C = Codec<kCodec>;
     using T = typename C::T;
-    // [kPen4][pitch] input ranks and output ranks (passes 2 and 3 work in place and share
-    // one table), then (list mode) [kPen4][nw] bitmaps of the cells with an output slot
-    extern __shared__ int s_rank4[];
-    __shared__ int s_any[kPen4];
+    // per pencil of the item: whether it holds any output slot, [pitch] input ranks and output
+    // ranks (passes 2 and 3 work in place and share one table), then (list mode) [nw] bitmaps
+    // of the cells with an output slot
+    extern __shared__ int s_any[];
     __shared__ long long s_w;
     const GridGeom& G = P.G;
     if (aborted(G.abort)) return;
@@ -351,10 +354,14 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
     const int nw = (nd + 31) >> 5;
     const int pitch = nd | 1;  // rank tables: the 16 pencils of a position lie in different banks
     const int64_t npen = G.N / nd;
-    int* s_rin = s_rank4;
-    int* s_rout = P.in_is_out ? s_rank4 : s_rank4 + kPen4 * pitch;
-    uint32_t* s_slot = reinterpret_cast<uint32_t*>(s_rank4 + (P.in_is_out ? 1 : 2) * kPen4 * pitch);
-    const int k = threadIdx.x >> 4;        // pencil; a warp holds pencils k and k^1
+    // 16-bit storage: one group per item (the loop over groups costs it registers: 15.1
+    // against 14.5 ms per bfloat16 step)
+    constexpr bool kMany = kCodec == 0;
+    const int npi = kMany ? 1 << P.lg_pen : kPen4;  // pencils of an item
+    int* s_rin = s_any + npi;
+    int* s_rout = P.in_is_out ? s_rin : s_rin + npi * pitch;
+    uint32_t* s_slot = reinterpret_cast<uint32_t*>(s_rout + npi * pitch);
+    const int k0 = threadIdx.x >> 4;       // pencil of kPen4; a warp holds pencils k0 and k0^1
     const int q = (threadIdx.x >> 2) & 3;  // velocity chunk (vz within the block)
     const int vy = threadIdx.x & 3;        // vx row of the chunk
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -367,14 +374,14 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
                 s_w = (long long)nx;
                 nx = atomicAdd(P.next, 1ull);
             }
-            if (threadIdx.x < kPen4) s_any[threadIdx.x] = 0;
+            for (int t = threadIdx.x; t < npi; t += blockDim.x) s_any[t] = 0;
             __syncthreads();
             const int64_t w = s_w;
             if (w >= P.item_base[G.nb]) break;
             pair = P.items[w];
         } else {
             if (!first) break;
-            if (threadIdx.x < kPen4) s_any[threadIdx.x] = 0;
+            for (int t = threadIdx.x; t < npi; t += blockDim.x) s_any[t] = 0;
             __syncthreads();
         }
         const int b = (int)(pair / P.groups);
@@ -387,10 +394,10 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
         const uint8_t din = P.in.dense[b], dout = P.out.dense[b];
         const bool all_in = (din & 1) && (!P.check_keep_in || (din & 2)), all_out = (dout & 1) != 0;
         const int64_t seg = (int64_t)b * G.RW;
-        for (int t = threadIdx.x; t < kPen4 * nd; t += blockDim.x) {
-            const int kk = P.dim == 0 ? t / nd : t & (kPen4 - 1);
-            const int i = P.dim == 0 ? t - kk * nd : t / kPen4;
-            const int64_t p = grp * kPen4 + kk;
+        for (int t = threadIdx.x; t < npi * nd; t += blockDim.x) {
+            const int kk = P.dim == 0 ? t / nd : t & (npi - 1);
+            const int i = P.dim == 0 ? t - kk * nd : kMany ? t >> P.lg_pen : t / kPen4;
+            const int64_t p = grp * npi + kk;
             int ri = -1, ro = -1;
             if (p < npen) {
                 int x;
@@ -421,13 +428,15 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
         __syncthreads();
         if constexpr (kList) {
             // which cells have an output slot, 32 per ballot
-            for (int j = warp; j < kPen4 * nw; j += kThreads4 / 32) {
+            for (int j = warp; j < npi * nw; j += kThreads4 / 32) {
                 const int kk = j / nw, c = ((j - kk * nw) << 5) + lane;
                 const unsigned bits = __ballot_sync(0xffffffffu, c < nd && s_rout[kk * pitch + c] >= 0);
                 if (lane == 0) s_slot[j] = bits;
             }
             __syncthreads();
         }
+        int k = k0;
+        do {
         if (!s_any[k] && !s_any[k ^ 1]) continue;  // warp-uniform
 
         const int bc[3] = {b % G.nbx, (b / G.nbx) % G.nby, b / (G.nbx * G.nby)};
@@ -607,6 +616,7 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
         push_emit(m, t0);
         push_emit(m + 1, t1);
         if constexpr (kLast) mass += (double)msum;
+        } while (kMany && (k += kPen4) < npi);
     }
     if constexpr (kLast) {
         for (int o = 16; o > 0; o >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
@@ -676,7 +686,16 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
                 if ((lo >= 0.0) != (hi >= 0.0)) vec = false;
             }
         }
-        const int per_cta = vec ? kPen4 : kPencils;
+        // An item's rank tables cost a fixed time (two global latencies and the barriers)
+        // before its walks start, so items of short pencils take several groups of them, as long
+        // as 16 items per SM are left.  3-pass step with one group, and up to 128, 256 and 512
+        // cells per item: shock 128x32x16 23.4, 22.4, 21.7, 21.2 ms; uniform 64x64x16 11.2, 10.8,
+        // 10.3, 10.3 ms (1024 cells would leave one CTA per SM).
+        int mult = 1;
+        while (vec && g->codec == 0 && 2 * mult * G.n[d] <= kItemCells && npen * G.nb / (kPen4 * 2 * mult) >= 16 * (int64_t)nsm) mult *= 2;
+        P.lg_pen = 4;
+        for (int i = mult; i > 1; i >>= 1) P.lg_pen++;
+        const int per_cta = vec ? kPen4 * mult : kPencils;
         P.groups = (npen + per_cta - 1) / per_cta;
         int64_t nblocks = P.groups * G.nb;
         if (nblocks > 0x7fffffffLL) return fail(g, VL_EINVAL, "3-pass form: grid too large");
@@ -686,9 +705,9 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
         const bool listed = vec && g->present < G.N * (int64_t)G.nb / 4 * 3;
         // rank tables (one when the pass works in place) and, listed, the slot bitmaps
         const int smem4 =
-            ((P.in_is_out ? 1 : 2) * kPen4 * (G.n[d] | 1) + (listed ? kPen4 * ((G.n[d] + 31) / 32) : 0)) * (int)sizeof(int);
+            per_cta * (1 + (P.in_is_out ? 1 : 2) * (G.n[d] | 1) + (listed ? (G.n[d] + 31) / 32 : 0)) * (int)sizeof(int);
         if (listed) {
-            k_pass_groups<<<(unsigned)((nblocks + 255) / 256), 256, 0, g->stream>>>(G, B.ubits, d, P.groups,
+            k_pass_groups<<<(unsigned)((nblocks + 255) / 256), 256, 0, g->stream>>>(G, B.ubits, d, per_cta, P.groups,
                                                                                     g->tile_flags);
             note_launch();
             launch_items_from_flags(g, P.groups, true);
