@@ -130,19 +130,16 @@ vl_status enqueue_step(Grid* g, StepArgs a, bool fused, bool graph, int64_t capa
     NvtxRange step_range("vl step");
     {
         NvtxRange range("union + index");
-        cudaMemsetAsync(ctr, 0, sizeof(StepCounters), g->stream);
-        launch_union(g, A, B);
+        launch_union(g, A, B, ctr);
         if (graph) {
-            launch_index(g, B);
-            launch_capacity_check(g, B, capacity, ctr);
+            launch_index(g, B, &A, ctr, capacity);
             cudaMemsetAsync(B.keepq, 0, (size_t)capacity * 4, g->stream);
         } else {
             int64_t total = 0;
-            vl_status st = layout_index(g, B, &total);
+            vl_status st = layout_index(g, B, &A, &total, ctr);
             if (st != VL_OK) return st;
             st = layout_ensure_pool(g, B, std::max<int64_t>(total, 1));
             if (st != VL_OK) return st;
-            cudaMemcpyAsync(&ctr->needed, B.base + g->geom.nb, 8, cudaMemcpyDeviceToDevice, g->stream);
             cudaMemsetAsync(B.keepq, 0, (size_t)std::max<int64_t>(total, 1) * 4, g->stream);
         }
     }

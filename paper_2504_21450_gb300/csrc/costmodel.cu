@@ -525,7 +525,7 @@ vl_status tile_features(Grid* g, int edge, float* feat, float* uni)
     }
     // the next layout's ubits become the 27-cell union of the state (the next step
     // rebuilds that layout anyway)
-    launch_union(g, g->lay[g->cur], g->lay[1 - g->cur]);
+    launch_union(g, g->lay[g->cur], g->lay[1 - g->cur], nullptr);
     // about eight CTAs per SM, parts of at least 16 ids
     const int split = (int)std::max<int64_t>(1, std::min<int64_t>((G.nb + 15) / 16, 152 * 8 / ntiles));
     const int ids = (G.nb + split - 1) / split;

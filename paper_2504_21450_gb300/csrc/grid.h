@@ -105,18 +105,20 @@ vl_status layout_ensure_pool(Grid* g, Layout& L, int64_t blocks);
 void layout_release_pool(Grid* g, Layout& L);
 // Like layout_ensure_pool, but keeps the L.total blocks the pool holds.
 vl_status layout_grow_pool(Grid* g, Layout& L, int64_t blocks);
-// Counts, offsets and dense flags of L from its ubits (woff, cnt, base, dense);
-// returns the total number of slots in *total (synchronises the stream).
-vl_status layout_index(Grid* g, Layout& L, int64_t* total);
-// next.ubits = 27-cell dilation of cur.kbits (periodic).
-void launch_union(Grid* g, const Layout& cur, Layout& next);
-// Device-only part of layout_index (no host synchronisation).
-void launch_index(Grid* g, Layout& L);
+// Counts, offsets and dense flags of L from its ubits (woff, cnt, base, dense), kcnt zeroed;
+// returns the total number of slots in *total and, with ctr, in ctr->needed (synchronises
+// the stream).  cur (optional): the state the step begins from, whose dense bit 1 is set from
+// its kcnt.
+vl_status layout_index(Grid* g, Layout& L, Layout* cur, int64_t* total, StepCounters* ctr);
+// Device-only part of layout_index (no host synchronisation).  Inside a captured sequence
+// (geom.abort set) a total above capacity sets the abort flag and ctr->error bit 3.
+void launch_index(Grid* g, Layout& L, Layout* cur, StepCounters* ctr, int64_t capacity);
+// next.ubits = 27-cell dilation of cur.kbits (periodic); ctr (optional) is zeroed.
+void launch_union(Grid* g, const Layout& cur, Layout& next, StepCounters* ctr);
 // next.kbits from the per-chunk keep flags; counts kept/dropped blocks and the FP64
-// mass of dropped blocks into ctr; sets next.dense bit 1 and next.kcnt; marks ctr done.
+// mass of dropped blocks into ctr; adds to next.kcnt; marks ctr done.  (Dense bit 1 is set
+// when the next step begins, by its index.)
 void launch_pack_keep(Grid* g, Layout& next, StepCounters* ctr);
-// Sets the abort flag and ctr->error bit 3 when L's slot total exceeds capacity.
-void launch_capacity_check(Grid* g, const Layout& L, int64_t capacity, StepCounters* ctr);
 vl_status set_blocks(Grid* g, int64_t nblocks, const int64_t* off, const uint16_t* ids,
                      const float* vals, int on_device);
 vl_status get_block_count(Grid* g, int64_t* n);

@@ -68,11 +68,12 @@ __global__ void k_seg_scan(const uint32_t* __restrict__ in, uint32_t* __restrict
     if (threadIdx.x == 0) seg_total[seg] = carry;
 }
 
-// base[s] = sum of seg_total[0..s), base[nseg] = grand total (64-bit); one CTA.
-__global__ void k_base_scan(const uint32_t* __restrict__ seg_total, int64_t* __restrict__ base,
-                            int64_t nseg, const int* abort)
+// base[s] = sum of seg_total[0..s), base[nseg] = grand total (64-bit); one CTA, which
+// finish(s, total of segment s) sees as well.
+template <class Finish>
+__device__ __forceinline__ int64_t base_scan(const uint32_t* __restrict__ seg_total, int64_t* __restrict__ base,
+                                             int64_t nseg, Finish&& finish)
 {
-    if (aborted(abort)) return;
     __shared__ unsigned long long wsum[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     unsigned long long carry = 0;
@@ -89,11 +90,50 @@ __global__ void k_base_scan(const uint32_t* __restrict__ seg_total, int64_t* __r
         }
         __syncthreads();
         unsigned long long pre = carry + (warp > 0 ? wsum[warp - 1] : 0ull);
-        if (i < nseg) base[i] = (int64_t)(pre + x - v);
+        if (i < nseg) {
+            base[i] = (int64_t)(pre + x - v);
+            finish(i, (uint32_t)v);
+        }
         carry += wsum[nw - 1];
         __syncthreads();
     }
     if (threadIdx.x == 0) base[nseg] = (int64_t)carry;
+    return (int64_t)carry;
+}
+
+__global__ void k_base_scan(const uint32_t* __restrict__ seg_total, int64_t* __restrict__ base,
+                            int64_t nseg, const int* abort)
+{
+    if (aborted(abort)) return;
+    base_scan(seg_total, base, nseg, [](int64_t, uint32_t) {});
+}
+
+// Offsets of a layout's segments, their dense flags (bit 0) and zeroed kept-block counts.  With
+// ctr: the slot total goes to ctr->needed, and a step whose pools were sized before it ran
+// (captured step sequences: capacity and abort) and whose union needs more slots than they
+// hold is skipped, like every later one, leaving the last complete state in its layout.
+// With kcnt_cur: dense bit 1 of the state the step begins from (all cells kept), whose
+// counts the last step's sparsity rule left.
+// One launch where a scan, two kernels for flags, the check and a memset were five: on the
+// smallest workload a step is launches (89 to 79 us per captured step of 8^3 cells).
+__global__ void k_index_finish(const uint32_t* __restrict__ cnt, int64_t* __restrict__ base,
+                               uint8_t* __restrict__ dense, uint32_t* __restrict__ kcnt,
+                               const uint32_t* __restrict__ kcnt_cur, uint8_t* __restrict__ dense_cur, int nb,
+                               int64_t N, int64_t capacity, int* abort, StepCounters* ctr)
+{
+    if (aborted(abort)) return;
+    const int64_t total = base_scan(cnt, base, nb, [&](int64_t b, uint32_t n) {
+        dense[b] = n == (uint32_t)N ? 1 : 0;
+        kcnt[b] = 0;
+        if (kcnt_cur && kcnt_cur[b] == (uint32_t)N) dense_cur[b] |= 2;
+    });
+    if (ctr && threadIdx.x == 0) {
+        ctr->needed = (long long)total;
+        if (abort && total > capacity) {
+            ctr->error |= 8;
+            *abort = 1;
+        }
+    }
 }
 
 __device__ __forceinline__ uint64_t word_mask(int nx, int w)
@@ -104,156 +144,153 @@ __device__ __forceinline__ uint64_t word_mask(int nx, int w)
     return top == 63 ? ~0ull : ((1ull << (top + 1)) - 1ull);
 }
 
-// One word of a row dilated by one cell along x with periodic wrap.
-__device__ __forceinline__ uint64_t xdilate(const uint64_t* row, int W, int nx, int w)
-{
-    uint64_t cur = row[w];
-    uint64_t prev = w > 0 ? row[w - 1] : 0ull;
-    uint64_t next = (w + 1 < W) ? row[w + 1] : 0ull;
-    uint64_t left = (cur << 1) | (prev >> 63);   // bit x receives bit x-1
-    uint64_t right = (cur >> 1) | (next << 63);  // bit x receives bit x+1
-    int last = nx - 1;
-    if (w == 0) left |= (row[last >> 6] >> (last & 63)) & 1ull;
-    if (w == (last >> 6)) right |= (row[0] & 1ull) << (last & 63);
-    return cur | left | right;
-}
-
 // next.ubits = union of cur.kbits over the 3x3x3 periodic neighbourhood (a block can
 // only arrive from a cell at most one step away along each axis, since |c| <= 1 per
-// sweep); next.wcount = popcount per word.
+// sweep); next.wcount = popcount per word.  The nine rows are joined before they are
+// dilated along x, which is then done once.  I: 32-bit indices wherever the words of all
+// bitmaps fit (64-bit divisions were most of the time: 111 us for 4.7 million words, 24 us
+// with both).  ctr (optional) is zeroed for the step that begins here, also when an
+// earlier step of a captured sequence has aborted.
+template <class I>
 __global__ void k_union(GridGeom G, const uint64_t* __restrict__ kin, uint64_t* __restrict__ uout,
-                        uint32_t* __restrict__ wcount)
+                        uint32_t* __restrict__ wcount, StepCounters* ctr)
 {
+    if (ctr && blockIdx.x == 0 && threadIdx.x == 0) *ctr = StepCounters{};
     if (aborted(G.abort)) return;
-    int64_t total = (int64_t)G.nb * G.RW;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t b = i / G.RW;
-        int64_t rw = i - b * G.RW;
-        int64_t row = rw / G.W;
-        int w = (int)(rw - row * G.W);
-        int y = (int)(row % G.n[1]);
-        int z = (int)(row / G.n[1]);
-        const uint64_t* seg = kin + b * G.RW;
-        uint64_t acc = 0;
-        for (int dz = -1; dz <= 1; dz++) {
-            int zz = wrapi(z + dz, G.n[2]);
-            for (int dy = -1; dy <= 1; dy++) {
-                int yy = wrapi(y + dy, G.n[1]);
-                const uint64_t* r = seg + ((int64_t)yy + (int64_t)G.n[1] * zz) * G.W;
-                acc |= xdilate(r, G.W, G.n[0], w);
+    const I total = (I)G.nb * (I)G.RW, RW = (I)G.RW, W = (I)G.W, ny = (I)G.n[1], nz = (I)G.n[2];
+    const int nx = G.n[0], last = (nx - 1) >> 6, top = (nx - 1) & 63;
+    for (I i = (I)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (I)gridDim.x * blockDim.x) {
+        const I b = i / RW, rw = i - b * RW;
+        const I row = W == 1 ? rw : rw / W;
+        const int w = (int)(rw - row * W);
+        const I z = row / ny, y = row - z * ny;
+        const I ys[3] = {y == 0 ? ny - 1 : y - 1, y, y + 1 == ny ? 0 : y + 1};
+        const I zs[3] = {z == 0 ? nz - 1 : z - 1, z, z + 1 == nz ? 0 : z + 1};
+        // this word of the nine rows, and the words that hold its neighbours along x
+        const int wl = w == 0 ? last : w - 1, wr = w == last ? 0 : w + 1;
+        const uint64_t* seg = kin + b * RW;
+        uint64_t cur = 0, left = 0, right = 0;
+#pragma unroll
+        for (int dz = 0; dz < 3; dz++)
+#pragma unroll
+            for (int dy = 0; dy < 3; dy++) {
+                const uint64_t* r = seg + (ys[dy] + ny * zs[dz]) * W;
+                cur |= r[w];
+                if (W > 1) {
+                    left |= r[wl];
+                    right |= r[wr];
+                }
             }
-        }
-        acc &= word_mask(G.n[0], w);
+        if (W == 1) left = right = cur;
+        // bit x receives bits x-1 and x+1; the row's first and last cells are neighbours
+        const uint64_t from_left = w == 0 ? (left >> top) & 1ull : left >> 63;
+        const uint64_t from_right = w == last ? (right & 1ull) << top : right << 63;
+        const uint64_t acc = (cur | cur << 1 | from_left | cur >> 1 | from_right) & word_mask(nx, w);
         uout[i] = acc;
         wcount[i] = (uint32_t)__popcll(acc);
     }
 }
 
-__global__ void k_dense_u(const uint32_t* __restrict__ cnt, uint8_t* __restrict__ dense, int nb,
-                          int64_t N, const int* abort)
+// dense bit 1 of a state that was set (kcnt: its blocks per id)
+__global__ void k_dense_k(const uint32_t* __restrict__ kcnt, uint8_t* __restrict__ dense, int nb, int64_t N)
 {
-    if (aborted(abort)) return;
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nb) dense[b] = (cnt[b] == (uint32_t)N) ? 1 : 0;
-}
-
-__global__ void k_dense_k(const uint32_t* __restrict__ kcnt, uint8_t* __restrict__ dense, int nb,
-                          int64_t N, const int* abort, StepCounters* ctr)
-{
-    if (aborted(abort)) return;
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < nb && kcnt[b] == (uint32_t)N) dense[b] |= 2;
-    if (ctr && b == 0) ctr->done = 1;
-}
-
-// Capacity check of a step whose pools were sized before it ran (captured step
-// sequences): when the union needs more slots than the pools hold, the step and every
-// later one are skipped, leaving the last complete state in its layout.
-__global__ void k_capacity(const int64_t* __restrict__ total, int64_t capacity, int* abort,
-                           StepCounters* ctr)
-{
-    if (aborted(abort)) return;
-    const int64_t t = *total;
-    ctr->needed = (long long)t;
-    if (t > capacity) {
-        ctr->error |= 8;
-        *abort = 1;
-    }
 }
 
 constexpr int kPackThreads = 256;
 
 // Sparsity rule: a slot of the new layout stays iff any of its four chunks had a value
 // >= threshold (the per-chunk flags are written by the sweep epilogue).  Removed blocks
-// add their FP64 mass (sum of the 64 averages) to the dropped mass.
+// add their FP64 mass (sum of the 64 averages) to the dropped mass.  A lane takes one cell of
+// a word, so that the flags of a word's slots, which lie side by side, are read in two
+// loads (a thread per word read them one after another: 142 us on 33.5 million slots, 57
+// now).  A warp takes `words` consecutive words of one block id (a multiple of 4, at most 32).
 template <int kCodec>
-__global__ void k_pack_keep(GridGeom G, LayoutView L, const uint8_t* __restrict__ keepq,
-                            uint64_t* __restrict__ kout, uint32_t* __restrict__ kcnt,
-                            StepCounters* __restrict__ ctr, int64_t chunks_per_seg)
+__global__ void __launch_bounds__(kPackThreads) k_pack_keep(GridGeom G, LayoutView L,
+                                                            const uint8_t* __restrict__ keepq,
+                                                            uint64_t* __restrict__ kout,
+                                                            uint32_t* __restrict__ kcnt,
+                                                            StepCounters* __restrict__ ctr, int words,
+                                                            unsigned ctas_per_seg)
 {
     if (aborted(G.abort)) return;
-    __shared__ unsigned long long s_kept[kPackThreads / 32], s_drop[kPackThreads / 32];
+    __shared__ unsigned s_kept[kPackThreads / 32], s_drop[kPackThreads / 32];
     __shared__ double s_mass[kPackThreads / 32];
-    const int64_t b = blockIdx.x / chunks_per_seg;
-    const int64_t rw = (blockIdx.x % chunks_per_seg) * kPackThreads + threadIdx.x;
-    unsigned long long kept = 0, drop = 0;
+    __shared__ uint32_t s_queue[kPackThreads / 32][4 * 64];  // ranks of removed blocks
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctr->done = 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned b = blockIdx.x / ctas_per_seg;
+    const int64_t rw0 = ((int64_t)(blockIdx.x - b * ctas_per_seg) * (kPackThreads / 32) + warp) * words;
+    const int nw = (int)max((int64_t)0, min((int64_t)words, G.RW - rw0));
+    const int64_t w0 = (int64_t)b * G.RW + rw0;
+    const int64_t bb = L.base[b];
+    const uint32_t cb = L.cnt[b];
+    // lane i < nw: word i
+    const uint64_t u_own = lane < nw ? L.ubits[w0 + lane] : 0ull;
+    const uint32_t o_own = lane < nw ? L.woff[w0 + lane] : 0u;
+    uint64_t k_own = 0;
+    unsigned kept = 0, drop = 0;
     double dmass = 0.0;
-    if (rw < G.RW) {
-        int64_t wi = b * G.RW + rw;
-        uint64_t u = L.ubits[wi];
-        uint64_t k = 0;
-        uint32_t wo = L.woff[wi];
-        int64_t bb = L.base[b];
-        uint32_t cb = L.cnt[b];
-        uint64_t rest = u;
-        while (rest) {
-            int bit = __ffsll((long long)rest) - 1;
-            rest &= rest - 1;
-            int64_t rank = (int64_t)wo + __popcll(u & ((1ull << bit) - 1ull));
-            int64_t slot = bb + rank;
-            uint32_t flags = *reinterpret_cast<const uint32_t*>(keepq + slot * 4);
-            if (flags) {
-                k |= 1ull << bit;
-                kept++;
-            } else {
-                drop++;
-                // the four chunks are loaded independently and each summed in FP32 (16
-                // values of one block: relative error ~1e-7 of a dropped block's mass);
-                // the chunk sums are accumulated in FP64
-                using T = typename Codec<kCodec>::T;
-                float cs[4];
+    const unsigned some = __ballot_sync(0xffffffffu, u_own != 0ull);
+    for (int i = 0; i < nw; i += 4) {
+        if (!((some >> i) & 0xfu)) continue;
+        // the flags of four words' slots in flight
+        uint32_t flags[4][2];
+        bool has[4][2];
+        uint32_t rank[4][2];
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const int64_t ci = bb * 4 + (int64_t)q * cb + rank;  // chunk index
-                    const float sc = kCodec ? L.scale[ci] : 1.0f;
-                    const T* p = static_cast<const T*>(L.pool) + ci * kChunk;
-                    float part[4] = {0.f, 0.f, 0.f, 0.f};
-                    if constexpr (kCodec == 0) {
-                        const float4* p4 = reinterpret_cast<const float4*>(p);
+        for (int j = 0; j < 4; j++) {
+            const uint64_t u = __shfl_sync(0xffffffffu, u_own, i + j);
+            const uint32_t o = __shfl_sync(0xffffffffu, o_own, i + j);
 #pragma unroll
-                        for (int j = 0; j < 4; j++) {
-                            const float4 v = p4[j];
-                            part[j] = (v.x + v.y) + (v.z + v.w);
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < kChunk; j++) part[j & 3] += Codec<kCodec>::dec(p[j], sc);
-                    }
-                    cs[q] = (part[0] + part[1]) + (part[2] + part[3]);
-                }
-                dmass += ((double)cs[0] + (double)cs[1]) + ((double)cs[2] + (double)cs[3]);
+            for (int h = 0; h < 2; h++) {
+                const int bit = lane + 32 * h;
+                has[j][h] = (u >> bit) & 1ull;
+                rank[j][h] = o + __popcll(u & ((1ull << bit) - 1ull));
+                flags[j][h] = has[j][h] ? *reinterpret_cast<const uint32_t*>(keepq + (bb + rank[j][h]) * 4) : 0u;
             }
         }
-        kout[wi] = k;
+        int nq = 0;  // removed blocks of these words
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            uint64_t k = 0;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const bool keep = flags[j][h] != 0u, out = has[j][h] && !keep;
+                const unsigned m = __ballot_sync(0xffffffffu, keep), d = __ballot_sync(0xffffffffu, out);
+                k |= (uint64_t)m << (32 * h);
+                kept += __popc(m);
+                if (out) s_queue[warp][nq + __popc(d & ((1u << lane) - 1u))] = rank[j][h];
+                nq += __popc(d);
+            }
+            if (lane == i + j) k_own = k;
+        }
+        drop += nq;
+        __syncwarp();
+        // their mass, four lanes per block (one vx row of every chunk each): a chunk's 16 values
+        // are summed in FP32 (relative error ~1e-7 of a removed block's mass), the chunk sums
+        // in FP64
+        for (int n = 0; n < nq; n += 8) {
+            const bool mine = n + (lane >> 2) < nq;
+            const uint32_t r = mine ? s_queue[warp][n + (lane >> 2)] : 0u;
+            Rows<kCodec> rows;
+            rows.load(L, bb * 4 + r, cb, lane & 3, mine);
+            float cs[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const float4 v = rows.get(q);
+                cs[q] = (v.x + v.y) + (v.z + v.w);
+                cs[q] += __shfl_xor_sync(0xffffffffu, cs[q], 1);
+                cs[q] += __shfl_xor_sync(0xffffffffu, cs[q], 2);
+            }
+            if (mine && (lane & 3) == 0) dmass += ((double)cs[0] + (double)cs[1]) + ((double)cs[2] + (double)cs[3]);
+        }
+        __syncwarp();
     }
+    if (lane < nw) kout[w0 + lane] = k_own;
     // CTA reduction, one atomic per CTA
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-        kept += __shfl_down_sync(0xffffffffu, kept, o);
-        drop += __shfl_down_sync(0xffffffffu, drop, o);
-        dmass += __shfl_down_sync(0xffffffffu, dmass, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) dmass += __shfl_down_sync(0xffffffffu, dmass, o);
     if (lane == 0) {
         s_kept[warp] = kept;
         s_drop[warp] = drop;
@@ -261,16 +298,16 @@ __global__ void k_pack_keep(GridGeom G, LayoutView L, const uint8_t* __restrict_
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long K = 0, D = 0;
+        unsigned K = 0, D = 0;
         double M = 0.0;
         for (int w = 0; w < kPackThreads / 32; w++) {
             K += s_kept[w];
             D += s_drop[w];
             M += s_mass[w];
         }
-        if (K) atomicAdd(&kcnt[b], (uint32_t)K);
-        if (K) atomicAdd(&ctr->kept, K);
-        if (D) atomicAdd(&ctr->dropped, D);
+        if (K) atomicAdd(&kcnt[b], K);
+        if (K) atomicAdd(&ctr->kept, (unsigned long long)K);
+        if (D) atomicAdd(&ctr->dropped, (unsigned long long)D);
         if (M != 0.0) atomicAdd(&ctr->dropped_mass, M);
     }
 }
@@ -454,12 +491,6 @@ void launch_base_scan(const uint32_t* seg_total, int64_t* base, int64_t nseg, cu
     k_base_scan<<<1, kScanThreads, 0, s>>>(seg_total, base, nseg, abort); note_launch();
 }
 
-void launch_capacity_check(Grid* g, const Layout& L, int64_t capacity, StepCounters* ctr)
-{
-    k_capacity<<<1, 1, 0, g->stream>>>(L.base + g->geom.nb, capacity, g->abort_flag, ctr);
-    note_launch();
-}
-
 vl_status layout_alloc_meta(Grid* g, Layout& L)
 {
     const GridGeom& G = g->geom;
@@ -528,12 +559,14 @@ vl_status layout_ensure_pool(Grid* g, Layout& L, int64_t blocks)
     return VL_OK;
 }
 
-void launch_index(Grid* g, Layout& L)
+void launch_index(Grid* g, Layout& L, Layout* cur, StepCounters* ctr, int64_t capacity)
 {
     const GridGeom& G = g->geom;
     launch_seg_scan(L.wcount, L.woff, L.cnt, G.RW, G.nb, g->stream, G.abort);
-    launch_base_scan(L.cnt, L.base, G.nb, g->stream, G.abort);
-    k_dense_u<<<nblk(G.nb, 256), 256, 0, g->stream>>>(L.cnt, L.dense, G.nb, G.N, G.abort); note_launch();
+    k_index_finish<<<1, kScanThreads, 0, g->stream>>>(L.cnt, L.base, L.dense, L.kcnt, cur ? cur->kcnt : nullptr,
+                                                      cur ? cur->dense : nullptr, G.nb, G.N, capacity,
+                                                      const_cast<int*>(G.abort), ctr);
+    note_launch();
 }
 
 vl_status layout_grow_pool(Grid* g, Layout& L, int64_t blocks)
@@ -565,10 +598,10 @@ vl_status layout_grow_pool(Grid* g, Layout& L, int64_t blocks)
     return VL_OK;
 }
 
-vl_status layout_index(Grid* g, Layout& L, int64_t* total)
+vl_status layout_index(Grid* g, Layout& L, Layout* cur, int64_t* total, StepCounters* ctr)
 {
     const GridGeom& G = g->geom;
-    launch_index(g, L);
+    launch_index(g, L, cur, ctr, INT64_MAX);
     cudaMemcpyAsync(g->host_scalar, L.base + G.nb, 8, cudaMemcpyDeviceToHost, g->stream);
     cudaError_t e = cudaStreamSynchronize(g->stream);
     if (e != cudaSuccess) return cuda_fail(g, e, "layout index");
@@ -577,25 +610,30 @@ vl_status layout_index(Grid* g, Layout& L, int64_t* total)
     return VL_OK;
 }
 
-void launch_union(Grid* g, const Layout& cur, Layout& next)
+void launch_union(Grid* g, const Layout& cur, Layout& next, StepCounters* ctr)
 {
     const GridGeom& G = g->geom;
-    int64_t total = (int64_t)G.nb * G.RW;
-    int blocks = (int)std::min<int64_t>(nblk(total, 256), 152 * 32);
-    k_union<<<blocks, 256, 0, g->stream>>>(G, cur.kbits, next.ubits, next.wcount); note_launch();
+    const int64_t total = (int64_t)G.nb * G.RW;
+    const int blocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 32);
+    // 32-bit indices also for the last stride past the end
+    if (total <= (int64_t)0x7fffffff)
+        k_union<uint32_t><<<blocks, 256, 0, g->stream>>>(G, cur.kbits, next.ubits, next.wcount, ctr);
+    else
+        k_union<int64_t><<<blocks, 256, 0, g->stream>>>(G, cur.kbits, next.ubits, next.wcount, ctr);
+    note_launch();
 }
 
 void launch_pack_keep(Grid* g, Layout& next, StepCounters* ctr)
 {
     const GridGeom& G = g->geom;
-    int64_t cps = (G.RW + kPackThreads - 1) / kPackThreads;
-    cudaMemsetAsync(next.kcnt, 0, (size_t)G.nb * 4, g->stream);
+    // 32 words a warp, fewer where a block id has fewer than a CTA's
+    const int words = (int)std::min<int64_t>(32, std::max<int64_t>(4, (G.RW + 7) / 8 / 4 * 4));
+    const int64_t per_cta = kPackThreads / 32 * words;
+    const int64_t cps = (G.RW + per_cta - 1) / per_cta;
     with_codec(g->codec, [&](auto c) {
         k_pack_keep<decltype(c)::value><<<(unsigned)(cps * G.nb), kPackThreads, 0, g->stream>>>(
-            G, next.view(), next.keepq, next.kbits, next.kcnt, ctr, cps);
+            G, next.view(), next.keepq, next.kbits, next.kcnt, ctr, words, (unsigned)cps);
     });
-    note_launch();
-    k_dense_k<<<nblk(G.nb, 256), 256, 0, g->stream>>>(next.kcnt, next.dense, G.nb, G.N, G.abort, ctr);
     note_launch();
 }
 
@@ -700,10 +738,10 @@ vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* 
     k_popcount<<<nblk((int64_t)words, 256), 256, 0, s>>>(L.ubits, L.wcount, (int64_t)words); note_launch();
     cudaMemcpyAsync(L.kbits, L.ubits, words * 8, cudaMemcpyDeviceToDevice, s);
     int64_t total = 0;
-    vl_status st = layout_index(g, L, &total);
+    vl_status st = layout_index(g, L, nullptr, &total, nullptr);
     if (st != VL_OK) return st;
     if (total != M) return fail(g, VL_EINVAL, "vl_set_blocks: duplicate block ids");
-    k_dense_k<<<nblk(G.nb, 256), 256, 0, s>>>(L.cnt, L.dense, G.nb, G.N, nullptr, nullptr); note_launch();
+    k_dense_k<<<nblk(G.nb, 256), 256, 0, s>>>(L.cnt, L.dense, G.nb, G.N); note_launch();
     st = layout_ensure_pool(g, L, std::max<int64_t>(M, 1));
     if (st != VL_OK) return st;
     const int64_t chunk = std::min<int64_t>(std::max<int64_t>(M, 1), (int64_t)1 << 22);  // 1 GiB of values
