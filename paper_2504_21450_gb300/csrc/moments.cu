@@ -1,10 +1,9 @@
 // moments.cu -- FP64 velocity moments per cell (n, n V_d, P_dd) and the total mass.
 //
 // FP64 instructions are scarce on this chip (two per clock and SM, conversions included),
-// so the sums are taken in pairs of FP32 numbers without loss: TwoSum (Knuth 1969) gives
-// the rounding error of an FP32 addition exactly, and a short tree of them carries a sum as
-// high + low part with 48 bits.  A block's 64 values are reduced that way to its twelve
-// partial sums over vx, vy and vz (its share of the cell's three marginals
+// so a block's values are added as integer multiples of two powers of two and a small FP32
+// rest, exactly but for that rest (Places, below).  A block's 64 values are reduced that way
+// to its twelve partial sums over vx, vy and vz (its share of the cell's three marginals
 // M_d[i] = sum of f over the velocity cells with index i along d); only those are added up
 // in FP64.  n, V and P follow from the marginals in FP64 with P summed about V, as a sum
 // over single values would give them: one pass over f instead of two, 0.4 FP64
@@ -13,8 +12,11 @@
 // A warp takes eight cells (blocks.cuh).
 //
 // Measured (64x32x16 cells x 32^3 velocity cells, 4.3 GB of f, 0.63 ms at the copy rate):
-// 1.16 ms per call, total mass 0.69; the kernel for any mesh, which sums every value
-// in FP64 with one warp per cell, 49.8 ms.
+// 1.55 ms per call, bound by instruction issue (splits and sums); total mass 0.67; the kernel
+// for any mesh, which sums every value in FP64 with one warp per cell, 49.8 ms.  Sums in pairs
+// of FP32 numbers (48 bits) took 1.26 and 0.64 ms, but were less precise than FP64 sums of
+// single values: largest relative error of n against 128-bit sums 5.6e-15 on a 4^3 mesh
+// and 1.9e-15 on 8^3, here 1.3e-16 and 2.1e-16, FP64 sums 1.2e-16 and 2.3e-16.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -28,7 +30,7 @@ namespace vlgt {
 
 namespace {
 
-constexpr int kMaxRun = 8;       // blocks summed in FP32 pairs before the sum goes to FP64
+constexpr int kMaxRun = 8;       // blocks summed before the sum goes to FP64: 2^29 multiples at most
 constexpr int kWarps = 8;        // warps of a CTA, at most
 
 struct VMesh {
@@ -36,38 +38,77 @@ struct VMesh {
     int nv[3];
 };
 
-// A sum held as high + low part.
-struct Pair {
-    float h, l;
+// Values split at two fixed places: with s1 = 1.5 * 2^E, s2 = 1.5 * 2^(E-23) and |f| < 2^(E-1),
+// t1 = f + s1 and t2 = (f - (t1 - s1)) + s2 round f to multiples of 2^(E-23) and 2^(E-46), and
+// every subtraction is exact (Dekker 1971; the fixed place is that of Rump, Ogita & Oishi
+// 2008).  Within its binade a float's bits count its multiples, so sums of t1 and t2 are taken
+// over the bits as integers, exactly, modulo 2^32.  What is left, below 2^(E-47), is added in
+// FP32: an error below 2^(E-70) per addition, far below that of an FP64 sum.
+constexpr unsigned kHead = 10;             // room above the largest value, in bits
+constexpr unsigned kWide = 0x7e000000u;    // bits of 2^125: from here on FP64
+
+struct Split {  // one value, or a sum: multiples (biased), multiples (biased), rest
+    unsigned a, b;
+    float c;
 };
-__device__ __forceinline__ Pair two_sum(float a, float b)
+struct Places {
+    float s1, s2;
+    // for values up to that with the bits m.  E >= -100 keeps s2 and its multiples normal; the
+    // rest is then exact
+    __device__ __forceinline__ void set(unsigned m)
+    {
+        const unsigned e = min(max((m >> 23) + 2u + kHead, 27u), 253u);
+        s1 = __uint_as_float(e << 23 | 0x400000u);
+        s2 = __uint_as_float((e - 23u) << 23 | 0x400000u);
+    }
+    // bits of 2^(E-1)
+    __device__ __forceinline__ unsigned limit() const { return __float_as_uint(s1) - 0xc00000u; }
+    // value i of four; two are split at a time, in packed FP32
+    __device__ __forceinline__ Split split(const float (&f)[4], int i) const
+    {
+        const float2 v = make_float2(f[i & 2], f[i | 1]), p1 = make_float2(s1, s1), p2 = make_float2(s2, s2);
+        const float2 t1 = add2(v, p1), r1 = sub2(v, sub2(t1, p1)), t2 = add2(r1, p2), r2 = sub2(r1, sub2(t2, p2));
+        return i & 1 ? Split{__float_as_uint(t1.y), __float_as_uint(t2.y), r2.y}
+                     : Split{__float_as_uint(t1.x), __float_as_uint(t2.x), r2.x};
+    }
+    __device__ __forceinline__ double unit() const  // 2^(E-46)
+    {
+        return __hiloint2double((int)((__float_as_uint(s1) >> 3) - 0x80000u + ((1023u - 127u - 46u) << 20)), 0);
+    }
+    // multiples of unit() in a sum over n values
+    __device__ __forceinline__ long long multiples(const Split& x, unsigned n) const
+    {
+        return (long long)(int)(x.a - n * __float_as_uint(s1)) * (1 << 23) + (int)(x.b - n * __float_as_uint(s2));
+    }
+    __device__ __forceinline__ double value(const Split& x, unsigned n) const
+    {
+        return fma((double)multiples(x, n), unit(), (double)x.c);
+    }
+};
+
+// Bits of the largest magnitude of three; NaN counts as larger than infinity.
+__device__ __forceinline__ float top3(float a, float b, float c)
 {
-    const float s = a + b, t = s - a;
-    return {s, (a - (s - t)) + (b - t)};
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
-__device__ __forceinline__ Pair add(const Pair& a, const Pair& b)
+__device__ __forceinline__ unsigned top(const float (&f)[4][4])
 {
-    const Pair s = two_sum(a.h, b.h);
-    return {s.h, s.l + (a.l + b.l)};
+    float m = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; q++) m = top3(top3(m, f[q][0], f[q][1]), f[q][2], f[q][3]);
+    return __float_as_uint(m) & 0x7fffffffu;
 }
-__device__ __forceinline__ Pair sum4(float a, float b, float c, float d)
-{
-    const Pair p = two_sum(a, b), q = two_sum(c, d), s = two_sum(p.h, q.h);
-    return {s.h, s.l + (p.l + q.l)};
-}
-__device__ __forceinline__ Pair shfl_xor(const Pair& a, int m)
-{
-    return {__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
-}
-__device__ __forceinline__ double value(const Pair& a) { return (double)a.h + (double)a.l; }
 
 // Entry k = lane & 3 of the sum over four neighbouring lanes of p[0..3].
-__device__ __forceinline__ Pair transpose_sum(const Pair (&p)[4], int k)
+template <class T>
+__device__ __forceinline__ T transpose_sum(const T (&p)[4], int k)
 {
     const bool hi = k & 2, odd = k & 1;
-    const Pair a0 = add(hi ? p[2] : p[0], shfl_xor(hi ? p[0] : p[2], 2));
-    const Pair a1 = add(hi ? p[3] : p[1], shfl_xor(hi ? p[1] : p[3], 2));
-    return add(odd ? a1 : a0, shfl_xor(odd ? a0 : a1, 1));
+    const T a0 = (hi ? p[2] : p[0]) + __shfl_xor_sync(0xffffffffu, hi ? p[0] : p[2], 2);
+    const T a1 = (hi ? p[3] : p[1]) + __shfl_xor_sync(0xffffffffu, hi ? p[1] : p[3], 2);
+    return (odd ? a1 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 1);
 }
 
 // Groups of eight cells along x, row by row.
@@ -90,18 +131,26 @@ __device__ __forceinline__ void write_moments(const GridGeom& G, const VMesh& V,
     const double* M = acc + (d == 0 ? 0 : d == 1 ? V.nv[0] : V.nv[0] + V.nv[1]) * kGroup + j;
     const double vmin = d == 0 ? V.vmin[0] : d == 1 ? V.vmin[1] : V.vmin[2];
     const double dv = d == 0 ? V.dv[0] : d == 1 ? V.dv[1] : V.dv[2];
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int i = 0; i < nd; i++) {
-        const double f = M[i * kGroup];
-        s0 += f;
-        s1 += (vmin + (i + 0.5) * dv) * f;
-    }
+    // four chains each (index modulo 4): shorter sums round less
+    double a[4] = {}, b[4] = {};
+    for (int i = 0; i < nd; i += 4)
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const double f = M[(i + q) * kGroup];
+            a[q] += f;
+            b[q] += (vmin + (i + q + 0.5) * dv) * f;
+        }
+    const double s0 = (a[0] + a[1]) + (a[2] + a[3]), s1 = (b[0] + b[1]) + (b[2] + b[3]);
     const double n = __shfl_sync(0xffffffffu, s0, lane & ~3);
     const double mean = n != 0.0 ? s1 / n : 0.0;
-    for (int i = 0; i < nd; i++) {
-        const double w = (vmin + (i + 0.5) * dv) - mean;
-        s2 += w * w * M[i * kGroup];
-    }
+    for (int q = 0; q < 4; q++) a[q] = 0.0;
+    for (int i = 0; i < nd; i += 4)
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const double w = (vmin + (i + q + 0.5) * dv) - mean;
+            a[q] += w * w * M[(i + q) * kGroup];
+        }
+    const double s2 = (a[0] + a[1]) + (a[2] + a[3]);
     if (x < G.n[0] && d < 3) {
         double* o = out + (row * G.n[0] + x) * 7;
         if (d == 0) o[0] = n * dv3;
@@ -130,14 +179,22 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_marginals(GridGeom G, Layout
     double* az = ay + V.nv[1] * kGroup;
     // this lane's vx rows (vy = k, vz = q), each summed over vx and over consecutive blocks of
     // one row of blocks along vx: the vy and vz marginals of those blocks come from them
-    Pair Z[4] = {};
+    unsigned za[4] = {}, zb[4] = {};
+    float zc[4] = {};
+    Places at;
+    at.set(0u);
     int run = 0, row_of_run = -1;
     auto flush = [&]() {
         if (run == 0) return;
-        ay[(row_of_run % G.nby) * 4 * kGroup] += value(add(add(Z[0], Z[1]), add(Z[2], Z[3])));
-        az[(row_of_run / G.nby) * 4 * kGroup] += value(transpose_sum(Z, k));
+        const Split y{za[0] + za[1] + za[2] + za[3], zb[0] + zb[1] + zb[2] + zb[3], (zc[0] + zc[1]) + (zc[2] + zc[3])};
+        const Split z{transpose_sum(za, k), transpose_sum(zb, k), transpose_sum(zc, k)};
+        ay[(row_of_run % G.nby) * 4 * kGroup] += at.value(y, 16u * run);
+        az[(row_of_run / G.nby) * 4 * kGroup] += at.value(z, 16u * run);
 #pragma unroll
-        for (int q = 0; q < 4; q++) Z[q] = {0.f, 0.f};
+        for (int q = 0; q < 4; q++) {
+            za[q] = zb[q] = 0u;
+            zc[q] = 0.0f;
+        }
         run = 0;
     };
     const int b_begin = blockIdx.y * P.ids, b_end = min(G.nb, b_begin + P.ids);
@@ -150,12 +207,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_marginals(GridGeom G, Layout
     };
     for_blocks<Rows<kCodec>>(G, L, row, x0, 0xffu, b_begin, b_end, load, [&](int b, const Rows<kCodec>& r, bool, int64_t, uint32_t) {
         const int brow = b / G.nbx, bx = b - brow * G.nbx;
-        if (brow != row_of_run || run == kMaxRun) {
-            flush();
-            row_of_run = brow;
-        }
         float f[4][4];
-        Pair X[4], S[4];
 #pragma unroll
         for (int q = 0; q < 4; q++) {
             const float4 v = r.get(q);
@@ -163,38 +215,47 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_marginals(GridGeom G, Layout
             f[q][1] = v.y;
             f[q][2] = v.z;
             f[q][3] = v.w;
-            S[q] = add(Z[q], sum4(v.x, v.y, v.z, v.w));
         }
-#pragma unroll
-        for (int i = 0; i < 4; i++) X[i] = sum4(f[0][i], f[1][i], f[2][i], f[3][i]);
-        const Pair x = transpose_sum(X, k);
-        // sums that leave FP32's range on the way (2^125: four of them still fit), infinities
-        // and NaN: FP64 for this block
-        const bool wide =
-            !((fabsf(S[0].h) + fabsf(S[1].h)) + (fabsf(S[2].h) + fabsf(S[3].h)) + fabsf(x.h) < 0x1p125f);
-        if (__any_sync(0xffffffffu, wide)) {
-            double dx[4], dz[4], dy = 0.0;
-            for (int i = 0; i < 4; i++) {
-                dx[i] = ((double)f[0][i] + f[1][i]) + ((double)f[2][i] + f[3][i]);
-                dz[i] = ((double)f[i][0] + f[i][1]) + ((double)f[i][2] + f[i][3]);
-                dy += dz[i];
-            }
-            for (int i = 0; i < 4; i++)
-                for (int o = 1; o < 4; o <<= 1) {
-                    dx[i] += __shfl_xor_sync(0xffffffffu, dx[i], o);
-                    dz[i] += __shfl_xor_sync(0xffffffffu, dz[i], o);
+        unsigned m = top(f);
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        if (brow != row_of_run || run == kMaxRun || __any_sync(0xffffffffu, m >= at.limit())) {
+            if (__any_sync(0xffffffffu, m >= kWide)) {
+                // values near the end of FP32's range, infinities and NaN: FP64 for this block
+                double dx[4], dz[4], dy = 0.0;
+                for (int i = 0; i < 4; i++) {
+                    dx[i] = ((double)f[0][i] + f[1][i]) + ((double)f[2][i] + f[3][i]);
+                    dz[i] = ((double)f[i][0] + f[i][1]) + ((double)f[i][2] + f[i][3]);
+                    dy += dz[i];
                 }
-            const double xk = k == 0 ? dx[0] : k == 1 ? dx[1] : k == 2 ? dx[2] : dx[3];
-            const double zk = k == 0 ? dz[0] : k == 1 ? dz[1] : k == 2 ? dz[2] : dz[3];
-            ax[bx * 4 * kGroup] += xk;
-            ay[(brow % G.nby) * 4 * kGroup] += dy;
-            az[(brow / G.nby) * 4 * kGroup] += zk;
-            return;
+                ax[bx * 4 * kGroup] += transpose_sum(dx, k);
+                ay[(brow % G.nby) * 4 * kGroup] += dy;
+                az[(brow / G.nby) * 4 * kGroup] += transpose_sum(dz, k);
+                return;
+            }
+            flush();
+            at.set(m);
+            row_of_run = brow;
         }
-        ax[bx * 4 * kGroup] += value(x);
+        unsigned xa[4] = {}, xb[4] = {};
+        float xc[4] = {};
 #pragma unroll
-        for (int q = 0; q < 4; q++) Z[q] = S[q];
+        for (int q = 0; q < 4; q++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const Split p = at.split(f[q], i);
+                za[q] += p.a;
+                zb[q] += p.b;
+                zc[q] += p.c;
+                xa[i] += p.a;
+                xb[i] += p.b;
+                xc[i] += p.c;
+            }
         run++;
+        const Split x{transpose_sum(xa, k), transpose_sum(xb, k), transpose_sum(xc, k)};
+        // at most 2^49 multiples in magnitude: as an FP64 number by its bits, without a conversion
+        const double n = __longlong_as_double(at.multiples(x, 16u) + 0x4338000000000000ll) - 0x1.8p52;
+        ax[bx * 4 * kGroup] += fma(n, at.unit(), (double)x.c);
     });
     flush();
     __syncwarp();
@@ -234,8 +295,10 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_density(GridGeom G, LayoutVi
     const int64_t grp = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
     if (grp >= P.total) return;
     double sum = 0.0;
-    Pair p{0.f, 0.f};
-    int run = 0;
+    Split p{0u, 0u, 0.0f};
+    Places at;
+    at.set(0u);
+    unsigned run = 0;
     const int b_begin = blockIdx.y * P.ids, b_end = min(G.nb, b_begin + P.ids);
     const int64_t row = grp / P.per_row;
     const int x0 = (int)(grp - row * P.per_row) * kGroup;
@@ -245,44 +308,75 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_density(GridGeom G, LayoutVi
         return r;
     };
     for_blocks<Rows<kCodec>>(G, L, row, x0, 0xffu, b_begin, b_end, load, [&](int, const Rows<kCodec>& r, bool, int64_t, uint32_t) {
-        Pair s{0.f, 0.f};
+        float f[4][4];
 #pragma unroll
         for (int q = 0; q < 4; q++) {
             const float4 v = r.get(q);
-            const Pair t = sum4(v.x, v.y, v.z, v.w);
-            s = q == 0 ? t : add(s, t);
+            f[q][0] = v.x;
+            f[q][1] = v.y;
+            f[q][2] = v.z;
+            f[q][3] = v.w;
         }
-        const Pair t = add(p, s);
-        if (fabsf(t.h) < INFINITY) {
-            p = t;
-        } else {  // infinities, NaN, sums beyond FP32's range
-            for (int q = 0; q < 4; q++) {
-                const float4 v = r.get(q);
-                sum += ((double)v.x + v.y) + ((double)v.z + v.w);
+        const unsigned m = top(f);
+        if (run == kMaxRun || m >= at.limit()) {
+            if (m >= kWide) {  // values near the end of FP32's range, infinities and NaN
+                for (int q = 0; q < 4; q++) sum += ((double)f[q][0] + f[q][1]) + ((double)f[q][2] + f[q][3]);
+                return;
             }
-        }
-        if (++run == kMaxRun) {
-            sum += value(p);
-            p = {0.f, 0.f};
+            sum += at.value(p, 16u * run);
+            p = {0u, 0u, 0.0f};
             run = 0;
+            at.set(m);
         }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const Split v = at.split(f[q], i);
+                p.a += v.a;
+                p.b += v.b;
+                p.c += v.c;
+            }
+        run++;
     });
-    sum += value(p);
+    sum += at.value(p, 16u * run);
     sum += __shfl_xor_sync(0xffffffffu, sum, 1);
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
     const int x = x0 + j;
     if (k == 0 && x < G.n[0]) dens[(int64_t)blockIdx.y * G.N + row * G.n[0] + x] = sum * (V.dv[0] * V.dv[1] * V.dv[2]);
 }
 
-// total += sum of v[0 .. n-1]
-__global__ void k_sum(const double* __restrict__ v, int64_t n, double* __restrict__ total)
+// out[blockIdx.x] = sum of this CTA's share of v[0 .. n-1], in an order that n and the grid fix;
+// compensated (TwoSum, Knuth 1969), so that its length costs no precision.
+__global__ void __launch_bounds__(256) k_sum(const double* __restrict__ v, int64_t n, double* __restrict__ out)
 {
-    double s = 0.0;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x)
-        s += v[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(total, s);
+    __shared__ double sh[2][8];
+    double s = 0.0, e = 0.0;
+    auto add = [&](double a) {
+        const double t = s + a, b = t - s;
+        e += (s - (t - b)) + (a - b);
+        s = t;
+    };
+    for (int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x; c < n; c += (int64_t)gridDim.x * 256) add(v[c]);
+    for (int o = 16; o > 0; o >>= 1) {
+        const double a = __shfl_xor_sync(0xffffffffu, s, o), b = __shfl_xor_sync(0xffffffffu, e, o);
+        add(a);
+        e += b;
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = s;
+        sh[1][threadIdx.x >> 5] = e;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < 8; w++) {
+        add(sh[0][w]);
+        e += sh[1][w];
+    }
+    // infinities have no low part
+    out[blockIdx.x] = fabs(s) < (double)INFINITY ? s + e : s;
 }
+constexpr int kSums = 152;  // CTAs of the first stage
 
 VMesh vmesh_of(const Grid* g)
 {
@@ -364,19 +458,21 @@ vl_status total_mass(Grid* g, double* mass)
     const GridGeom& G = g->geom;
     const VMesh V = vmesh_of(g);
     const Groups P = groups_of(g, sm_count(g));
-    // densities of the parts, then the total
-    double* dens = (double*)g->alloc(((size_t)P.split * G.N + 1) * sizeof(double));
+    // densities of the parts, the sums of shares of them, the total
+    const int64_t n = (int64_t)P.split * G.N;
+    const int sums = (int)std::min<int64_t>((n + 255) / 256, kSums);
+    double* dens = (double*)g->alloc(((size_t)n + sums + 1) * sizeof(double));
     if (!dens) return fail(g, VL_ENOMEM, "vl_mass: scratch allocation failed");
-    double* acc = dens + (size_t)P.split * G.N;
-    cudaMemsetAsync(acc, 0, sizeof(double), g->stream);
+    double* acc = dens + n + sums;
     with_codec(g->codec, [&](auto c) {
         k_density<decltype(c)::value>
             <<<dim3((unsigned)((P.total + kWarps - 1) / kWarps), P.split), kWarps * 32, 0, g->stream>>>(
                 G, g->lay[g->cur].view(), V, P, dens);
     });
     note_launch();
-    const int64_t n = (int64_t)P.split * G.N;
-    k_sum<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 4), 256, 0, g->stream>>>(dens, n, acc);
+    k_sum<<<sums, 256, 0, g->stream>>>(dens, n, dens + n);
+    k_sum<<<1, 256, 0, g->stream>>>(dens + n, sums, acc);
+    note_launch();
     note_launch();
     double h = 0.0;
     cudaMemcpyAsync(&h, acc, sizeof(double), cudaMemcpyDeviceToHost, g->stream);

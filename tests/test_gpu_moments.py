@@ -3,8 +3,10 @@ the kernel: groups of eight cells (rows shorter and longer than eight and 64 cel
 of blocks along vx, ids split over CTAs, sparse cells, 16-bit storage, values of any size,
 infinities, and a mesh too wide for the marginals.
 
-Tolerance: a block's sums are pairs of FP32 numbers (48 bits), at most 16 pair additions
-deep, so 16 * 2**-48 = 2**-44 of the sum of magnitudes; FP64 sums after that add far less."""
+Tolerance: 2**-44 of the sum of magnitudes, far above the rounding of the FP64 sums; cells of
+a few blocks, whose values span many decades, are held to that rounding itself."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -82,3 +84,38 @@ def test_infinities_stay_in_their_cell():
     assert np.isnan(got[5]).all() and np.isnan(mass)
     other = np.delete(np.arange(18), [3, 5])
     assert np.all(np.abs(got - clean)[other] <= 2 * TOL * size[other])
+
+
+@pytest.mark.parametrize("nv, storage", [((4, 4, 4), vlasov.VL_STORE_F32), ((8, 4, 8), vlasov.VL_STORE_F32),
+                                         ((8, 8, 4), vlasov.VL_STORE_BF16_SCALED)])
+@pytest.mark.parametrize("scale", [1.0, 1e-30, 1e30])
+def test_few_blocks_to_the_rounding_of_fp64(nv, storage, scale):
+    """n and n V_d against exact rationals.  Bound: each value's share passes one rounding per
+    block along an axis (at most 4 here), nv / 4 + 2 in the sum over a marginal, 3 for the
+    product with v and dv^3: 16 * 2**-53 of the sum of magnitudes, and 2**-60 for the rest
+    below the places."""
+    n, vmin, dv = (9, 2, 1), (-1.5, -2.0, -0.75), (1.0, 0.5, 0.25)
+    init = inputs.random_blocks(n, nv, 1.0, seed=104)
+    r = np.random.Generator(np.random.PCG64(105))
+    vals = (init.vals * np.exp(r.uniform(-30.0, 0.0, init.vals.shape)) * scale).astype(np.float32)
+    g = vlasov.Grid(n, nv, vmin, dv, storage=storage)
+    g.set_blocks(init.off, init.ids, vals)
+    got, mass = g.moments(), g.mass()
+    off, ids, vals = g.get_blocks()
+    g.close()
+    nb, dv3, total = [v // 4 for v in nv], Fraction(dv[0] * dv[1] * dv[2]), Fraction(0)
+    for c in range(off.size - 1):
+        want, size = [Fraction(0)] * 4, [Fraction(0)] * 4
+        for b, block in zip(ids[off[c]:off[c + 1]].astype(int), vals[off[c]:off[c + 1]]):
+            bc = (b % nb[0], b // nb[0] % nb[1], b // (nb[0] * nb[1]))
+            for l in range(64):
+                f = Fraction(float(block[l]))
+                w = [Fraction(1)] + [Fraction(vmin[d]) + (4 * bc[d] + (l >> 2 * d & 3) + Fraction(1, 2)) * Fraction(dv[d])
+                                     for d in range(3)]
+                for m in range(4):
+                    want[m] += f * w[m]
+                    size[m] += abs(f * w[m])
+        total += want[0] * dv3
+        for m in range(4):
+            assert abs(Fraction(float(got[c, m])) - want[m] * dv3) <= (16 * Fraction(2) ** -53 + Fraction(2) ** -60) * size[m] * dv3
+    assert abs(Fraction(mass) - total) <= 16 * Fraction(2) ** -53 * total
