@@ -11,8 +11,8 @@
 // the tile's blocks after the 27-cell union); summed over tiles this sizes the pools.
 // It never touches f: it changes only how much memory a captured sequence reserves.
 //
-// All reductions are deterministic (fixed summation order, FP64 accumulators), so a
-// training run is reproducible bit for bit.
+// All reductions are deterministic (fixed summation order; FP64, or pairs of FP32 numbers
+// whose values are added in FP64), so a training run is reproducible bit for bit.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -283,7 +283,9 @@ struct PairSum {
 // The 4801 sums over samples are what bounds an epoch.  FP64 instructions are scarce (two
 // per clock and SM), so a thread keeps its ten sums as FP32 pairs over the CTA's samples
 // and only their values are added in FP64.  Measured with 5696 samples: 44 us an epoch;
-// one thread per parameter with FP64 sums over all samples took 833.
+// one thread per parameter with FP64 sums over all samples took 833.  The gradient is the
+// same to its last bit's rounding (largest error against FP64 autograd, relative to the
+// largest entry, 500 to 20000 samples: 3.5e-8 to 4.5e-8 either way).
 template <bool kDirect>
 __global__ void __launch_bounds__(kMlpThreads) k_mlp_slab(const float* __restrict__ params,
                                                           const float* __restrict__ x,
