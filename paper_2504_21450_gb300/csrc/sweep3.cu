@@ -34,8 +34,7 @@ struct PassArgs {
     int dim;            // physical axis of this pass
     int check_keep_in;  // 1: read only present blocks of `in`
     int in_is_out;      // 1: `in` and `out` are the same layout (passes 2 and 3, in place)
-    double cs;          // dt / dx_dim
-    double vmin, dv;    // velocity mesh along dim
+    const float4* walk; // WalkConst (g, A, B, up) per velocity index along dim
     int last;           // last pass: keep flags and mass
     float thr;
     uint8_t* keepq;
@@ -122,7 +121,8 @@ __global__ void __launch_bounds__(kThreads3) k_pass(PassArgs P)
     int bc[3] = {b % G.nbx, (b / G.nbx) % G.nby, b / (G.nbx * G.nby)};
     int within[3] = {v & 3, (v >> 2) & 3, v >> 4};
     int iv = bc[P.dim] * 4 + within[P.dim];
-    const WalkConst kc = walk_const((P.vmin + (iv + 0.5) * P.dv) * P.cs);
+    const float4 w = P.walk[iv];
+    const WalkConst kc{w.x, w.y, w.z, w.w != 0.0f};
     const bool up = kc.up != 0;
     // the warp's velocity cells move the same way unless the block straddles v_d = 0
     const bool uni = __all_sync(0xffffffffu, up) || __all_sync(0xffffffffu, !up);
@@ -390,6 +390,17 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
         const int b = (int)(pair / P.groups);
         const int64_t grp = pair - (int64_t)b * P.groups;
         if (!kList && P.out.cnt[b] == 0) continue;  // CTA-uniform; a listed pair has slots
+        // The sweep constants of the row's four cells, from the table that the fused form reads.
+        // Worked out in FP64 by each thread for each group of pencils (about 60 instructions, at
+        // two per clock and SM) they were what short pencils waited for: 10.24 against 9.00 ms per
+        // step on 64x64x16 cells of the uniform workload, 21.07 against 18.03 on 128x32x16 of the
+        // shock, 14.49 against 13.25 in bfloat16, and 62 against 43 us on 8x8x8.
+        const int bc = P.dim == 0 ? b % G.nbx : P.dim == 1 ? (b / G.nbx) % G.nby : b / (G.nbx * G.nby);
+        float4 kc[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) kc[i] = P.walk[bc * 4 + (P.dim == 0 ? i : P.dim == 1 ? vy : q)];
+        const bool up = kc[0].w != 0.0f;
+        const WalkConst2 kp[2] = {pack_const(kc[0], kc[1]), pack_const(kc[2], kc[3])};
         // The dense flags are read once per item, and for y and z pencils neighbouring lanes take
         // neighbouring cells along x, whose bitmap words are the same (one lookup per cell in
         // pencil order, each with its own flag: 23.87 against 23.45 ms per step on 128x32x16
@@ -442,16 +453,6 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
         do {
         if (!s_any[k] && !s_any[k ^ 1]) continue;  // warp-uniform
 
-        const int bc[3] = {b % G.nbx, (b / G.nbx) % G.nby, b / (G.nbx * G.nby)};
-        WalkConst kc[4];
-    #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const int within = P.dim == 0 ? i : (P.dim == 1 ? vy : q);
-            const int iv = bc[P.dim] * 4 + within;
-            kc[i] = walk_const((P.vmin + (iv + 0.5) * P.dv) * P.cs);
-        }
-        const bool up = kc[0].up != 0;
-        const WalkConst2 kp[2] = {pack_const(kc[0], kc[1]), pack_const(kc[2], kc[3])};
         const bool uni = __all_sync(0xffffffffu, up) || __all_sync(0xffffffffu, !up);
 
         const int64_t cin = (int64_t)P.in.base[b] * 4 + (int64_t)q * P.in.cnt[b];    // chunk of rank 0
@@ -680,9 +681,7 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
         P.dim = d;
         P.check_keep_in = j == 0 ? 1 : 0;
         P.in_is_out = j == 0 ? 0 : 1;
-        P.cs = a.c_scale[d];
-        P.vmin = g->vmesh.vmin[d];
-        P.dv = g->vmesh.dv[d];
+        P.walk = a.walk + d * a.nvmax;
         P.last = j == 2 ? 1 : 0;
         P.thr = (float)g->threshold;
         P.keepq = B.keepq;
@@ -699,7 +698,8 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
         if (d == 0 || (d == 1 && g->codec)) {
             const int nbd = d == 0 ? G.nbx : G.nby;
             for (int bi = 0; bi < nbd && vec; bi++) {
-                const double lo = P.vmin + (4 * bi + 0.5) * P.dv, hi = P.vmin + (4 * bi + 3.5) * P.dv;
+                const double vmin = g->vmesh.vmin[d], dv = g->vmesh.dv[d];
+                const double lo = vmin + (4 * bi + 0.5) * dv, hi = vmin + (4 * bi + 3.5) * dv;
                 if ((lo >= 0.0) != (hi >= 0.0)) vec = false;
             }
         }
