@@ -308,11 +308,11 @@ __device__ __forceinline__ WalkConst2 pack_const(const float4& p, const float4& 
 // add every 2, a min or max every cycle), so of the packed forms only those that save
 // instructions by more than they cost are used, and the halved d0 takes one multiply out.
 // Cycles per push and scheduler with four warps (a loop of pushes): 37.6 before both
-// changes, 35.6 with them.  kForm: which of the two remaining fmas is written as two scalar
-// ones (0 none, 1 the limiter's, 2 the face value's); which is fastest depends on the
-// registers of the loop around it.  Plane-batched kernel: 1 (13.63 against 13.95 ms, 64x64x32
-// cells of the uniform workload); 3-pass kernel, 64x64x16 cells: 0 in FP32 (11.28 ms, form 1
-// 11.59, 2 11.34), 2 in bfloat16 (14.61 ms, form 0 14.80, 1 15.00).
+// changes, 35.6 with them.  kForm 1: the limiter's fma is written as two scalar
+// ones; whether that pays depends on the registers of the loop around it.  Plane-batched
+// kernel: 13.63 against 13.95 ms (64x64x32 cells of the uniform workload); 3-pass kernel: 8.99
+// against 9.00 (64x64x16 cells), 17.88 against 18.03 (shock, 128x32x16), 12.93 against 13.21
+// (bfloat16, 64x64x16).
 template <bool kLimiter, int kForm = 0>
 struct Walk2 {
     float2 a1, a2, l1, l2, h0, o3;
@@ -327,8 +327,7 @@ struct Walk2 {
         const float2 dn = sub2(a, a1);
         const float2 h = mul2(l1, make_float2(0.5f, 0.5f));
         const float2 t = sub2(l2, dn);
-        const float2 e = kForm == 2 ? make_float2(fmaf(t.x, 1.0f / 12.0f, h.x), fmaf(t.y, 1.0f / 12.0f, h.y))
-                                    : fma2(t, make_float2(1.0f / 12.0f, 1.0f / 12.0f), h);
+        const float2 e = fma2(t, make_float2(1.0f / 12.0f, 1.0f / 12.0f), h);
         float2 d1, out;
         if (kLimiter) {
             d1.x = copysignf(fmaxf(min_xorsign_abs(e.x, l1.x), 0.0f), l1.x);

@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
         load(0, t0);
         load(1 % nd, t1);
 
-        Walk2<kLim, kCodec != 0 ? 2 : 0> s[2];  // cells (0, 1) and (2, 3) of the row, packed
+        Walk2<kLim, 1> s[2];  // cells (0, 1) and (2, 3) of the row, packed
         s[0].reset();
         s[1].reset();
         float msum = 0.0f;
