@@ -357,8 +357,8 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
     const int nw = (nd + 31) >> 5;
     const int pitch = nd | 1;  // rank tables: the 16 pencils of a position lie in different banks
     const int64_t npen = G.N / nd;
-    // 16-bit storage: one group per item (the loop over groups costs it registers: 15.1
-    // against 14.5 ms per bfloat16 step)
+    // 16-bit storage: one group per item (the loop over groups costs it registers: 13.6
+    // against 13.2 ms per bfloat16 step)
     constexpr bool kMany = kCodec == 0;
     const int npi = kMany ? 1 << P.lg_pen : kPen4;  // pencils of an item
     int* s_rin = s_any + npi;
@@ -705,9 +705,10 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
         }
         // An item's rank tables cost a fixed time (two global latencies and the barriers)
         // before its walks start, so items of short pencils take several groups of them, as long
-        // as 16 items per SM are left.  3-pass step with one group, and up to 128, 256 and 512
-        // cells per item: shock 128x32x16 23.4, 22.4, 21.7, 21.2 ms; uniform 64x64x16 11.2, 10.8,
-        // 10.3, 10.3 ms (1024 cells would leave one CTA per SM).
+        // as 16 items per SM are left.  3-pass step with up to 256, 512 and 1024 cells per
+        // item: shock 128x32x16 18.2, 18.0, 21.0 ms (1024 cells leave one CTA per SM); uniform
+        // 64x64x16 8.87, 9.00, 9.00.  With one group, before the sweep constants came from a
+        // table, 23.4 and 11.2 against 21.2 and 10.3.
         int mult = 1;
         while (vec && g->codec == 0 && 2 * mult * G.n[d] <= kItemCells && npen * G.nb / (kPen4 * 2 * mult) >= 16 * (int64_t)nsm) mult *= 2;
         P.lg_pen = 4;
