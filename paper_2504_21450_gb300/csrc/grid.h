@@ -185,7 +185,8 @@ struct StepArgs {
 // Host-side fault injection for tests: true when the environment variable VLGT_FAULT
 // lists `what` (comma-separated).  "timeout": the fused kernel reports staging waits
 // that are not complete at their first poll as overdue (VL_ETIMEOUT) -- they still
-// complete, so no copy is left in flight.
+// complete, so no copy is left in flight.  "slow_slots": the plane-batched kernel's staging
+// warps take 50 us longer before they write the output slots of a batch.
 bool fault_requested(const char* what);
 
 // NVTX range over a host scope (phases of a step show up in a timeline profiler; the

@@ -116,10 +116,16 @@ struct Gt3Args {
     const int64_t* npairs;   // their number
     uint8_t* keepq;
     StepCounters* ctr;
-    int report_late;    // testing hook: a staging wait not complete at its first poll is
-                        // reported as overdue (VL_ETIMEOUT), then waited for
+    int testing;        // testing hooks, see kTestLate and kTestSlots
     uint64_t* cta_done; // optional [gridDim.x]: %globaltimer when the CTA ran out of work
 };
+
+// Testing hooks (Gt3Args::testing).  kTestLate: a staging wait not complete at its first poll
+// is reported as overdue (VL_ETIMEOUT), then waited for.  kTestSlots: the staging warps sleep
+// before they write a batch's output slots, so that a sweeping warp which were not made to
+// wait for them would read those of an earlier batch.
+constexpr int kTestLate = 1, kTestSlots = 2;
+constexpr unsigned kTestSlotsNs = 50000;  // a batch is swept in about 5 us
 
 __device__ __forceinline__ unsigned su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -325,7 +331,11 @@ __device__ __forceinline__ void item_tables(const Gt3Args& P, const Item& it, It
 // Staging of batch k of an item (planes kNB k .. kNB k + 2 of its stream) into buffer
 // g & 1, g = the CTA's running batch index; run by the kNS staging threads (sl = 0..127),
 // one staged row per thread, and every staging thread arrives on the batch's barrier
-// once its copies have landed.  Contiguous runs of a row go by TMA bulk copies; the short
+// once its copies have landed.  What staging threads write themselves (an item's description
+// and tables, zeroed cells, output slots) is published by arrivals that release it: a
+// cp.async arrival does not release its thread's own stores, so each staging warp adds one
+// plain arrival, the last thing it does for a batch, after its lanes' stores (__syncwarp).
+// Nothing that a sweeping warp reads is written after it.  Contiguous runs of a row go by TMA bulk copies; the short
 // run where a dense row wraps around the periodic grid (kShortRun cells or fewer) goes by
 // 16-byte cp.async copies instead: the SM's bulk-copy unit takes a roughly fixed time per
 // request, and these runs would add half as many requests again.  The chunk scale of each staged cell goes into the scale table with a 4-byte
@@ -363,6 +373,18 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
     const float* ipool = static_cast<const float*>(P.in.pool);
     auto plane_of = [&](int s) { return it.up2 ? s - kHalo : n2 + 2 - s; };
     auto out_of = [&](int s) { return it.up2 ? s - kFirst : n2 + 4 - s; };
+    // output slots of the tile cells of a sparse next layout, two threads per tile row: their
+    // bitmap words are read first, so that they come in while the copies are issued
+    const int oj = sw / (2 * kT), orr = (sw >> 1) - oj * kT;
+    const bool slots = !it.dense_out && sw < nj * 2 * kT && kNB * k + oj >= kFirst;
+    uint64_t ouw = 0ull;
+    uint32_t oow = 0u;
+    if (slots && orr < it.er) {
+        const int64_t row = (int64_t)rowpart(P.ar, it.tr0 + orr, ny) + rowpart(a2, out_of(kNB * k + oj), ny);
+        const int64_t wi = (int64_t)it.b * G.RW + row * G.W + (it.tx0 >> 6);
+        ouw = P.out.ubits[wi];
+        oow = P.out.woff[wi];
+    }
     if constexpr (kCodec != 0) {
         using T = typename Codec<kCodec>::T;
         const T* cpool = static_cast<const T*>(P.in.pool) + it.ibase;  // codes of rank 0
@@ -454,7 +476,6 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
         // arrival (the phase also waits for every staging thread's arrival below)
         if (kA0X && it.dense_in && sl == 0)
             bar_add_tx(bar, (unsigned)(nj * kLines * bulk_cells(t) * kChunk * sizeof(T)));
-        cp_arrive(bar);
     } else if (it.dense_in) {
         // the batch's bulk-copy bytes, announced once (the copies of the other staging
         // threads may complete before or after it; the phase also waits for every staging
@@ -477,12 +498,9 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
                 }
             }
         }
-        cp_arrive(bar);
     } else {
         // runs of present cells (consecutive slots) as bulk copies, each announced to the
-        // barrier before it is issued; absent cells are zeroed.  Each staging thread
-        // arrives after announcing its bytes, so the phase cannot end before every
-        // announcement.
+        // barrier before it is issued; absent cells are zeroed
         if (sw < nj * kLines) {
             const int j = sw / kLines, rho = t.r0 + sw - j * kLines;
             const int pz = wrapi(plane_of(kNB * k + j), n2);
@@ -527,32 +545,24 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
                 }
             }
         }
-        bar_arrive(bar);
     }
-    // output slots of the tile cells of a sparse next layout, two threads per tile row
-    if (!it.dense_out && sw < nj * 2 * kT) {
-        const int j = sw / (2 * kT), rr = (sw >> 1) - j * kT;
-        const int s = kNB * k + j;
-        if (s >= kFirst) {
-            const int zo = out_of(s);
-            int* orow = &S.orank[slot][j][rr * kT];
-            uint64_t uw = 0ull;
-            uint32_t ow = 0u;
-            if (rr < it.er) {
-                const int64_t row = (int64_t)rowpart(P.ar, it.tr0 + rr, ny) + rowpart(a2, zo, ny);
-                const int64_t wi = (int64_t)it.b * G.RW + row * G.W + (it.tx0 >> 6);
-                uw = P.out.ubits[wi];
-                ow = P.out.woff[wi];
-            }
+    if (slots) {
+        if (P.testing & kTestSlots) __nanosleep(kTestSlotsNs);
+        int* orow = &S.orank[slot][oj][orr * kT];
 #pragma unroll
-            for (int i8 = 0; i8 < kT / 2; i8++) {
-                const int i = (sw & 1) * (kT / 2) + i8;
-                const int bit = (it.tx0 + i) & 63;  // the 16 cells share one bitmap word
-                const bool has = i < it.ex && ((uw >> bit) & 1ull);
-                orow[i] = has ? (int)(ow + __popcll(uw & ((1ull << bit) - 1ull))) : -1;
-            }
+        for (int i8 = 0; i8 < kT / 2; i8++) {
+            const int i = (sw & 1) * (kT / 2) + i8;
+            const int bit = (it.tx0 + i) & 63;  // the 16 cells share one bitmap word
+            const bool has = i < it.ex && ((ouw >> bit) & 1ull);
+            orow[i] = has ? (int)(oow + __popcll(ouw & ((1ull << bit) - 1ull))) : -1;
         }
     }
+    // every thread arrives after announcing its bytes, so the phase cannot end before every
+    // announcement; deferred until its cp.async copies land where there may be any
+    if (kCodec != 0 || it.dense_in) cp_arrive(bar);
+    else bar_arrive(bar);
+    __syncwarp();
+    if ((sl & 31) == 0) bar_arrive(bar);
 }
 
 // The staging warps: they run up to two batches ahead of the sweeping warps, across
@@ -585,7 +595,7 @@ __device__ __forceinline__ void stage_loop(const Gt3Args& P, Gt3Smem& S, int sl,
         if (S.work[par] >= nwork) {
             // nothing more to stage: the phase completes and tells the sweeping warps to end
             bar_arrive(&S.bar[g & 1u]);
-            if (sl == 0) bar_arrive(&S.bar[g & 1u]);
+            if ((sl & 31) == 0) bar_arrive(&S.bar[g & 1u]);
             return;
         }
         const Item& it = S.item[par];
@@ -595,9 +605,6 @@ __device__ __forceinline__ void stage_loop(const Gt3Args& P, Gt3Smem& S, int sl,
             named_sync(kBarStage, kNS);
             late = S.late != 0;
             if (late) break;
-            // the plain arrival publishes the item's description and tables; the others
-            // may be deferred until a thread's copies land
-            if (sl == 0) bar_arrive(&S.bar[g & 1u]);
             stage_batch<kCodec, kA0X>(P, S, it, S.tab[par], k, g, sl);
         }
     }
@@ -631,7 +638,7 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
 
     if (tid == 0) {
         for (int i = 0; i < 2; i++) {
-            bar_init(&S.bar[i], kNS + 1);         // every staging thread, and one plain arrival
+            bar_init(&S.bar[i], kNS + kNS / 32);  // every staging thread, and each staging warp
             bar_init(&S.empty[i], kNC / 32);      // every sweeping warp
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -652,7 +659,7 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
     // a staged batch, or the end of the work list
     auto wait_staged = [&](unsigned g) {
         const unsigned slot = g & 1u, parity = (g >> 1) & 1u;
-        if (P.report_late && tid == 0 && !bar_test(&S.bar[slot], parity)) atomicOr(&P.ctr->error, 4);
+        if ((P.testing & kTestLate) && tid == 0 && !bar_test(&S.bar[slot], parity)) atomicOr(&P.ctr->error, 4);
         if (!bar_wait_bounded(&S.bar[slot], parity)) {
             atomicOr(&P.ctr->error, 4);
             S.abort = 1;
@@ -923,7 +930,7 @@ vl_status launch_gt3_dense(const GridGeom& G, const LayoutView& in, const Layout
     P.npairs = npairs;
     P.keepq = nullptr;
     P.ctr = ctr;
-    P.report_late = 0;
+    P.testing = 0;
     P.cta_done = nullptr;
     Grid tmp;  // launch helper needs the device and the stream only
     tmp.dev.device = device;
@@ -975,7 +982,7 @@ vl_status run_gt3(Grid* g, const StepArgs& a)
     P.npairs = g->item_base + G.nb;
     P.keepq = B.keepq;
     P.ctr = a.ctr;
-    P.report_late = fault_requested("timeout") ? 1 : 0;
+    P.testing = (fault_requested("timeout") ? kTestLate : 0) | (fault_requested("slow_slots") ? kTestSlots : 0);
     P.cta_done = a.stamp_ctas ? g->cta_done : nullptr;
     record_sweep_event(a.ev0, g->stream, a.ev_node);
     const bool a0x = a.order[0] == 0;
