@@ -851,7 +851,8 @@ __global__ void __launch_bounds__(kNT, 1) k_gt3(Gt3Args P)
         }
         gb += (unsigned)nbatch;
     }
-    double m = (double)msum;
+    // the sum runs over all items of the CTA: its low part goes with it
+    double m = (double)msum - (double)mcomp;
     for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
     if (lane == 0 && m != 0.0) atomicAdd(&P.ctr->mass, m);
     if (P.cta_done && tid == 0) P.cta_done[blockIdx.x] = now_ns();
