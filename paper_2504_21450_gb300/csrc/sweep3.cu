@@ -248,6 +248,16 @@ constexpr int kPen4 = 16;
 constexpr int kThreads4 = kPen4 * 16;
 constexpr int kBatch4 = 8;
 constexpr int kItemCells = 512;  // FP32: cells of an item's pencils end to end, at most (or one pencil)
+// Limit of a launch's dynamic shared memory, set before every launch: list mode has a few bytes
+// of static memory besides, so that even tables of exactly 48 KiB (several extents ask for
+// those) are refused without it.  One value for all launches, since the limit belongs to the
+// kernel: a grid that lowered it to its own size would take it from another grid's thread.
+// Most that an item asks for: kPen4 pencils of kMaxLine cells, two rank tables and the bitmaps,
+// 133312 bytes; several groups of pencils at most 131072 (up to 8192 pencils of one cell or
+// 4096 of two; longer pencils less).
+constexpr int kSmem4 = 133 * 1024;
+static_assert(kPen4 * (1 + 2 * (kMaxLine | 1) + (kMaxLine + 31) / 32) * 4 <= kSmem4, "tables of the longest pencils");
+static_assert((kPen4 * kItemCells) * (1 + 2 + 1) * 4 <= kSmem4, "tables of the shortest pencils");
 
 template <int kCodec>
 __device__ __forceinline__ void load4(const typename Codec<kCodec>::T* p, float sc, float (&o)[4])
@@ -741,7 +751,7 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
                                      : (P.last ? k_pass4<false, kc, true, kL> : k_pass4<false, kc, false, kL>);
                 };
                 auto kern = listed ? pick(std::true_type{}) : pick(std::false_type{});
-                if (smem4 > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem4);
+                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem4);
                 int per_sm = 0;
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads4, smem4);
                 const int64_t nct = listed ? std::min<int64_t>(nblocks, (int64_t)nsm * std::max(per_sm, 1)) : nblocks;
@@ -756,7 +766,8 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
                 auto kern = a.limiter ? k_pass<true, kc> : k_pass<false, kc>;
                 // 16-bit storage: per-chunk maxima of the pencils
                 const int smem = kc ? kPencils * 4 * G.n[d] * (int)sizeof(unsigned) : 0;
-                if (smem > 0) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                if (kc) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kPencils * 4 * kMaxLine * (int)sizeof(unsigned));
                 kern<<<(unsigned)nblocks, kThreads3, smem, g->stream>>>(P);
             }
         });
