@@ -150,7 +150,7 @@ void launch_blocks_out(Grid* g, const Layout& L, const Window& W, const int64_t*
 void launch_blocks_in(Grid* g, const Layout& L, const Window& W, const int64_t* off, const uint32_t* start,
                       const float* vals);
 // Marks the listed blocks of every cell in ubits; err |= 2 (id out of range), 4 (ids not
-// strictly increasing within a cell).
+// strictly increasing within a cell).  Does nothing when err has bit 0 (invalid offsets).
 void launch_mark_cells(Grid* g, const int64_t* off, const uint16_t* ids, int64_t M, uint64_t* ubits, int* err);
 // ---- moments.cu ------------------------------------------------------------
 // The velocity mesh is narrow enough for queue_moments, which is queue_cell_moments for

@@ -242,14 +242,15 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_blocks_in(GridGeom G, Layout
 }
 
 // Checks the lists (err bit 1: id out of range, bit 2: ids not strictly increasing within
-// a cell) and marks their blocks in ubits; one warp per cell.  The offsets may be invalid
-// (reported elsewhere): every access stays within the M listed blocks.
+// a cell) and marks their blocks in ubits; one warp per cell.  Nothing is walked when the
+// offsets are known to be invalid (err bit 0, from the check queued before): each cell could
+// then claim the whole list, and the work would be cells times blocks.
 __global__ void __launch_bounds__(kWarps * 32) k_mark_cells(GridGeom G, const int64_t* __restrict__ off,
                                                             const uint16_t* __restrict__ ids, int64_t M,
                                                             uint64_t* __restrict__ ubits, int* __restrict__ err)
 {
     const int64_t c = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
-    if (c >= G.N) return;
+    if (c >= G.N || (*(volatile const int*)err & 1)) return;
     const int64_t lo = max((int64_t)0, off[c]), hi = min(M, off[c + 1]);
     const int x = (int)(c % G.n[0]);
     uint64_t* words = ubits + c / G.n[0] * G.W + (x >> 6);
