@@ -407,6 +407,14 @@ size_t warp_bytes(const Grid* g)
     return (size_t)(g->vmesh.nv[0] + g->vmesh.nv[1] + g->vmesh.nv[2]) * kGroup * sizeof(double);
 }
 constexpr size_t kSmemCta = 100 * 1024;  // two CTAs per SM
+// The limit of a launch belongs to the kernel, not to the grid, and can be lowered: it is set
+// to the same value before every launch, so that a grid on another host thread never takes it
+// away between the two calls.
+template <class Kernel>
+void raise_smem(Kernel kern)
+{
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCta);
+}
 
 int sm_count(const Grid* g)
 {
@@ -440,12 +448,12 @@ vl_status queue_moments(Grid* g, double* d_out, void** scratch)
     with_codec(g->codec, [&](auto c) {
         constexpr int kc = decltype(c)::value;
         auto kern = P.split > 1 ? k_marginals<kc, true> : k_marginals<kc, false>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        raise_smem(kern);
         kern<<<dim3(ctas, P.split), warps * 32, smem, g->stream>>>(G, L, V, P, parts ? parts : d_out);
     });
     note_launch();
     if (P.split > 1) {
-        cudaFuncSetAttribute(k_join_marginals, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        raise_smem(k_join_marginals);
         k_join_marginals<<<ctas, warps * 32, smem, g->stream>>>(G, V, P, parts, d_out);
         note_launch();
     }
