@@ -351,7 +351,7 @@ vl_status vl_translate_dense_noalloc(const vl_space_desc* space, const vl_vmesh_
  * vl_mlp_forward: y[s] for n samples x[n][8] (device).
  * vl_mlp_gradient: dL/dparams into grad (device, VL_MLP_NPARAM) and L into *loss
  *   (device double), sums over samples in a fixed order (reproducible): L in FP64, the
- *   gradient in pairs of FP32 numbers (48 bits) over parts of the samples and in FP64
+ *   gradient in triples of FP32 numbers (72 bits) over parts of the samples and in FP64
  *   over the parts.
  * vl_mlp_train_step: one full-batch Adam step (beta1 VL_MLP_BETA1, beta2 VL_MLP_BETA2,
  *   eps VL_MLP_EPS, bias-corrected; step counts from 1) on params with the moment

@@ -11,7 +11,7 @@
 // the tile's blocks after the 27-cell union); summed over tiles this sizes the pools.
 // It never touches f: it changes only how much memory a captured sequence reserves.
 //
-// All reductions are deterministic (fixed summation order; FP64, or pairs of FP32 numbers
+// All reductions are deterministic (fixed summation order; FP64, or triples of FP32 numbers
 // whose values are added in FP64), so a training run is reproducible bit for bit.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -257,23 +257,40 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_forward(const float* __rest
     }
 }
 
-// A sum of products held as high + low part: the product's rounding error by an fma, the
-// sum's by TwoSum (Knuth 1969), both exact, so the sum carries 48 bits.
-struct PairSum {
-    float h, l;
-    __device__ __forceinline__ void add(float p, float e)
+// A sum held as three FP32 numbers: a product's rounding error by an fma and the rounding
+// errors of the high and middle sums by TwoSum (Knuth 1969), all exact, so that only the low
+// sum rounds, 2^-72 below the value.  Its FP64 value is rounded once (2^-53), where an FP64
+// sum of the same products rounds each time.  What lies below FP32's smallest number, 2^-149,
+// is lost; the gradient is FP32.
+struct TripleSum {
+    float h, m, l;
+    static __device__ __forceinline__ float two_sum(float a, float b, float& err)
     {
-        const float s = h + p, t = s - h;
-        l += ((h - (s - t)) + (p - t)) + e;
-        h = s;
+        const float s = a + b, t = s - a;
+        err = (a - (s - t)) + (b - t);
+        return s;
+    }
+    __device__ __forceinline__ void add(float p)
+    {
+        float r, r1;
+        h = two_sum(h, p, r);
+        m = two_sum(m, r, r1);
+        l += r1;
     }
     __device__ __forceinline__ void add_product(float a, float b)
     {
-        const float p = a * b;
-        add(p, fmaf(a, b, -p));
+        const float p = a * b, e = fmaf(a, b, -p);
+        float r, r1, r2;
+        h = two_sum(h, p, r);
+        m = two_sum(m, r, r1);
+        m = two_sum(m, e, r2);
+        l += r1 + r2;
     }
-    // an overflowed sum has no low part
-    __device__ __forceinline__ double value() const { return fabsf(h) < INFINITY ? (double)h + (double)l : (double)h; }
+    // an overflowed sum has no lower parts
+    __device__ __forceinline__ double value() const
+    {
+        return fabsf(h) < INFINITY ? (double)h + ((double)m + (double)l) : (double)h;
+    }
 };
 
 // Gradient of L = (1/n) sum (y - t)^2 and the sum of squares over samples blockIdx.x * per
@@ -281,11 +298,12 @@ struct PairSum {
 // dL/d(pre-activation) of layer 2 is d2, of layer 1 d1; the ReLU passes the gradient where
 // its output > 0.
 // The 4801 sums over samples are what bounds an epoch.  FP64 instructions are scarce (two
-// per clock and SM), so a thread keeps its ten sums as FP32 pairs over the CTA's samples
-// and only their values are added in FP64.  Measured with 5696 samples: 44 us an epoch;
-// one thread per parameter with FP64 sums over all samples took 833.  The gradient is the
-// same to its last bit's rounding (largest error against FP64 autograd, relative to the
-// largest entry, 500 to 20000 samples: 3.5e-8 to 4.5e-8 either way).
+// per clock and SM), so a thread keeps its ten sums as FP32 triples over the CTA's samples
+// and only their values are added in FP64.  Measured with 5696 samples: 60 us an epoch; one
+// thread per parameter with FP64 sums over all samples took 833, and pairs (48 bits, less
+// than FP64's 53) 48.  The gradient is the same to its last bit's rounding (largest error
+// against FP64 autograd, relative to the largest entry, 500 to 20000 samples: 3.5e-8 to 4.5e-8
+// in all three).
 template <bool kDirect>
 __global__ void __launch_bounds__(kMlpThreads) k_mlp_slab(const float* __restrict__ params,
                                                           const float* __restrict__ x,
@@ -301,7 +319,7 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_slab(const float* __restric
     // this thread's parameters: W2 rows 2 j2, 2 j2 + 1, columns 4 k4 .. + 3; W1 entry tid; and of
     // threads 0 .. 192 one of b1, b2, w3, b3
     const int j2 = 2 * (tid >> 4), k4 = 4 * (tid & 15);
-    PairSum g2[2][4] = {}, g1 = {}, g0 = {};
+    TripleSum g2[2][4] = {}, g1 = {}, g0 = {};
     double err = 0.0;  // of the sample whose output this thread has (first lane of a warp)
     const int64_t begin = (int64_t)blockIdx.x * per, end = min(n, begin + per);
     for (int64_t s0 = begin; s0 < end; s0 += kMlpBatch) {
@@ -349,14 +367,14 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_slab(const float* __restric
 #pragma unroll
                 for (int k = 0; k < 4; k++) g2[i][k].add_product(dv[i], hv[k]);
             g1.add_product(S.d1[s][tid / kIn], S.x[s][tid % kIn]);
-            if (tid < kH) g0.add(S.d1[s][u], 0.0f);
-            else if (tid < 2 * kH) g0.add(S.d2[s][u], 0.0f);
+            if (tid < kH) g0.add(S.d1[s][u]);
+            else if (tid < 2 * kH) g0.add(S.d2[s][u]);
             else if (tid < 3 * kH) g0.add_product(S.dy[s], S.h2[s][u]);
-            else if (tid == 3 * kH) g0.add(S.dy[s], 0.0f);
+            else if (tid == 3 * kH) g0.add(S.dy[s]);
         }
         __syncthreads();  // the batch's activations are no longer read
     }
-    auto put = [&](int p, const PairSum& g) {
+    auto put = [&](int p, const TripleSum& g) {
         if (kDirect) grad[p] = (float)g.value();
         else part[(int64_t)blockIdx.x * (kP + 1) + p] = g.value();
     };
