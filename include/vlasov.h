@@ -350,9 +350,9 @@ vl_status vl_translate_dense_noalloc(const vl_space_desc* space, const vl_vmesh_
  * W2[64][64], b2[64], w3[64], b3.  Loss L = (1/n) sum_s (y_s - t_s)^2.
  * vl_mlp_forward: y[s] for n samples x[n][8] (device).
  * vl_mlp_gradient: dL/dparams into grad (device, VL_MLP_NPARAM) and L into *loss
- *   (device double), sums over samples in a fixed order (reproducible): L in FP64, the
- *   gradient in triples of FP32 numbers (72 bits) over parts of the samples and in FP64
- *   over the parts.
+ *   (device double), sums over samples in an order that n alone fixes (reproducible, on
+ *   any GPU): L in FP64, the gradient in triples of FP32 numbers (72 bits) over parts of
+ *   the samples and in FP64 over the parts.
  * vl_mlp_train_step: one full-batch Adam step (beta1 VL_MLP_BETA1, beta2 VL_MLP_BETA2,
  *   eps VL_MLP_EPS, bias-corrected; step counts from 1) on params with the moment
  *   arrays adam_m, adam_v (device, VL_MLP_NPARAM each, zero before step 1); *loss

@@ -463,8 +463,10 @@ __global__ void k_capacity_sum(const float* __restrict__ y, int64_t n, double ma
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Workspace of a training step, of vl_mlp_workspace_bytes: the loss, the gradient, then
-// the CTAs' parts.  About one kB per sample, so that a part covers about 38 samples or, with
-// more than 38 samples per SM, there is one part per SM.
+// the CTAs' parts.  About one kB per sample, so that a part covers about 38 samples, up to
+// kMaxParts parts: one per SM of a GB300, a constant, so that the order of the sums and with it
+// their last bits depend on the number of samples alone, and not on the GPU.
+constexpr int kMaxParts = 152;
 constexpr size_t kWsGrad = 256, kWsParts = kWsGrad + ((size_t)kP * 4 + 255) / 256 * 256;
 
 size_t train_ws_bytes(int64_t n)
@@ -482,11 +484,8 @@ vl_status queue_gradient(const float* params, const float* x, const float* t, in
     double* loss = copy_loss ? reinterpret_cast<double*>(ws) : loss_out;
     float* grad = grad_out ? grad_out : reinterpret_cast<float*>(ws + kWsGrad);
     double* part = reinterpret_cast<double*>(ws + kWsParts);
-    int device = 0, nsm = 0;
-    cudaGetDevice(&device);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
     const int64_t room = (int64_t)((train_ws_bytes(n) - kWsParts) / ((kP + 1) * sizeof(double)));
-    const int64_t most = std::max<int64_t>(1, std::min<int64_t>(nsm, room));
+    const int64_t most = std::max<int64_t>(1, std::min<int64_t>(kMaxParts, room));
     const int64_t per = (n + most - 1) / most;
     const int parts = (int)((n + per - 1) / per);
     const AdamArgs none{};

@@ -389,13 +389,17 @@ VMesh vmesh_of(const Grid* g)
     return V;
 }
 
-Groups groups_of(const Grid* g, int nsm)
+// Sixteen warps for each of a GB300's SMs; a constant, so that the parts, and with them the last
+// bits of the sums over parts, depend on the grid alone, and not on the GPU.
+constexpr int64_t kWantWarps = 152 * 16;
+
+Groups groups_of(const Grid* g)
 {
     const GridGeom& G = g->geom;
     Groups P;
     P.per_row = (G.n[0] + kGroup - 1) / kGroup;
     P.total = (int64_t)P.per_row * G.R;
-    const Parts s = parts_of(G.nb, P.total, (int64_t)nsm * 16, 64);  // a part has marginals to join
+    const Parts s = parts_of(G.nb, P.total, kWantWarps, 64);  // a part has marginals to join
     P.split = s.split;
     P.ids = s.ids;
     return P;
@@ -416,13 +420,6 @@ void raise_smem(Kernel kern)
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCta);
 }
 
-int sm_count(const Grid* g)
-{
-    int n = 0;
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, g->dev.device);
-    return std::max(n, 1);
-}
-
 }  // namespace
 
 bool moments_fit(const Grid* g) { return warp_bytes(g) <= kSmemCta; }
@@ -433,7 +430,7 @@ vl_status queue_moments(Grid* g, double* d_out, void** scratch)
     const GridGeom& G = g->geom;
     const LayoutView L = g->lay[g->cur].view();
     const VMesh V = vmesh_of(g);
-    const Groups P = groups_of(g, sm_count(g));
+    const Groups P = groups_of(g);
     const size_t wb = warp_bytes(g);
     const int warps = (int)std::max<size_t>(1, std::min<size_t>(kWarps, kSmemCta / wb));
     const unsigned ctas = (unsigned)((P.total + warps - 1) / warps);
@@ -465,7 +462,7 @@ vl_status total_mass(Grid* g, double* mass)
 {
     const GridGeom& G = g->geom;
     const VMesh V = vmesh_of(g);
-    const Groups P = groups_of(g, sm_count(g));
+    const Groups P = groups_of(g);
     // densities of the parts, the sums of shares of them, the total
     const int64_t n = (int64_t)P.split * G.N;
     const int sums = (int)std::min<int64_t>((n + 255) / 256, kSums);
