@@ -463,7 +463,9 @@ __global__ void __launch_bounds__(NT, 1) k_fused(FusedArgs P)
         };
         auto keep_flags = [&](int s) {  // per-chunk keep flags of the plane completed at s
             const int zo = out_of(s);
-            if (s < FIRST || zo < 0 || zo >= n2) return;
+            // a caller that wants no flags gives none to write; its threshold of +infinity does
+            // not keep out a value that is infinite itself
+            if (!P.keepq || s < FIRST || zo < 0 || zo >= n2) return;
             const unsigned* km = kb + (s % 3) * 16;
             for (int c = ltid; c < TX * TY; c += NLD) {
                 int j = c / TX, i = c - j * TX;
