@@ -335,11 +335,12 @@ __device__ __forceinline__ void item_tables(const Gt3Args& P, const Item& it, It
 // and tables, zeroed cells, output slots) is published by arrivals that release it: a
 // cp.async arrival does not release its thread's own stores, so each staging warp adds one
 // plain arrival, the last thing it does for a batch, after its lanes' stores (__syncwarp).
-// Nothing that a sweeping warp reads is written after it.  Contiguous runs of a row go by TMA bulk copies; the short
-// run where a dense row wraps around the periodic grid (kShortRun cells or fewer) goes by
-// 16-byte cp.async copies instead: the SM's bulk-copy unit takes a roughly fixed time per
-// request, and these runs would add half as many requests again.  The chunk scale of each staged cell goes into the scale table with a 4-byte
-// cp.async copy (0 for an absent cell).  With sweep 0 along x the row's codes are packed
+// Nothing that a sweeping warp reads is written after it.  Contiguous runs of a row go by TMA
+// bulk copies; the short run where a dense row wraps around the periodic grid (kShortRun cells
+// or fewer) goes by 16-byte cp.async copies instead: the SM's bulk-copy unit takes a roughly
+// fixed time per request, and these runs would add half as many requests again.  The chunk
+// scale of each staged cell goes into the scale table with a 4-byte cp.async copy (0 for an
+// absent cell).  With sweep 0 along x the row's codes are packed
 // at one end of the row (kCodesHi) by bulk copies per contiguous run: sweep 0 walks
 // towards that end and writes its FP32 result two cells behind the one it reads, which
 // overwrites only codes read at least three positions earlier.  Otherwise the 32 bytes of
@@ -373,18 +374,6 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
     const float* ipool = static_cast<const float*>(P.in.pool);
     auto plane_of = [&](int s) { return it.up2 ? s - kHalo : n2 + 2 - s; };
     auto out_of = [&](int s) { return it.up2 ? s - kFirst : n2 + 4 - s; };
-    // output slots of the tile cells of a sparse next layout, two threads per tile row: their
-    // bitmap words are read first, so that they come in while the copies are issued
-    const int oj = sw / (2 * kT), orr = (sw >> 1) - oj * kT;
-    const bool slots = !it.dense_out && sw < nj * 2 * kT && kNB * k + oj >= kFirst;
-    uint64_t ouw = 0ull;
-    uint32_t oow = 0u;
-    if (slots && orr < it.er) {
-        const int64_t row = (int64_t)rowpart(P.ar, it.tr0 + orr, ny) + rowpart(a2, out_of(kNB * k + oj), ny);
-        const int64_t wi = (int64_t)it.b * G.RW + row * G.W + (it.tx0 >> 6);
-        ouw = P.out.ubits[wi];
-        oow = P.out.woff[wi];
-    }
     if constexpr (kCodec != 0) {
         using T = typename Codec<kCodec>::T;
         const T* cpool = static_cast<const T*>(P.in.pool) + it.ibase;  // codes of rank 0
@@ -546,21 +535,35 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
             }
         }
     }
-    if (slots) {
+    // every thread arrives after announcing its bytes, so the phase cannot end before every
+    // announcement; deferred until its cp.async copies land where there may be any
+    if (kCodec != 0 || it.dense_in) cp_arrive(bar);
+    else bar_arrive(bar);
+    // output slots of the tile cells of a sparse next layout, two threads per tile row.  (Read
+    // before the copies are issued, with the thread's arrival after the stores, the bitmap
+    // words cost registers on every state: 8.73 against 8.71 ms a sweep in bfloat16, 64x64x16
+    // cells of the uniform workload, 15.99 against 15.94 on 128x32x16 of the shock.)
+    const int oj = sw / (2 * kT), orr = (sw >> 1) - oj * kT;
+    if (!it.dense_out && sw < nj * 2 * kT && kNB * k + oj >= kFirst) {
+        uint64_t uw = 0ull;
+        uint32_t ow = 0u;
+        if (orr < it.er) {
+            const int64_t row = (int64_t)rowpart(P.ar, it.tr0 + orr, ny) + rowpart(a2, out_of(kNB * k + oj), ny);
+            const int64_t wi = (int64_t)it.b * G.RW + row * G.W + (it.tx0 >> 6);
+            uw = P.out.ubits[wi];
+            ow = P.out.woff[wi];
+        }
         if (P.testing & kTestSlots) __nanosleep(kTestSlotsNs);
         int* orow = &S.orank[slot][oj][orr * kT];
 #pragma unroll
         for (int i8 = 0; i8 < kT / 2; i8++) {
             const int i = (sw & 1) * (kT / 2) + i8;
             const int bit = (it.tx0 + i) & 63;  // the 16 cells share one bitmap word
-            const bool has = i < it.ex && ((ouw >> bit) & 1ull);
-            orow[i] = has ? (int)(oow + __popcll(ouw & ((1ull << bit) - 1ull))) : -1;
+            const bool has = i < it.ex && ((uw >> bit) & 1ull);
+            orow[i] = has ? (int)(ow + __popcll(uw & ((1ull << bit) - 1ull))) : -1;
         }
     }
-    // every thread arrives after announcing its bytes, so the phase cannot end before every
-    // announcement; deferred until its cp.async copies land where there may be any
-    if (kCodec != 0 || it.dense_in) cp_arrive(bar);
-    else bar_arrive(bar);
+    // publishes what the warp's lanes have written, the slots above among them
     __syncwarp();
     if ((sl & 31) == 0) bar_arrive(bar);
 }
