@@ -233,7 +233,8 @@ __host__ __device__ inline WalkConst walk_const(double c)
 // and w are <= 0 and the cell sends g a, as CW84's flattening prescribes; otherwise
 // |u| = |minmod(d1, 2 d0)| and |w| = |minmod(d0, 2 d1)|.
 // d0 is held halved (h0), so that 2 d0 is 4 h0 and minxs(d0, 2 d1) is twice
-// minxs(h0, d1): scalings by powers of two, which are exact.
+// minxs(h0, d1): scalings by powers of two, which are exact (below 2^-125 a halving may drop
+// the last bit, 2^-149).
 template <bool kLimiter>
 struct Walk {
     float a1, a2;  // a_{p-1}, a_{p-2}
@@ -312,7 +313,7 @@ __device__ __forceinline__ WalkConst2 pack_const(const float4& p, const float4& 
 // ones; whether that pays depends on the registers of the loop around it.  Plane-batched
 // kernel: 13.63 against 13.95 ms (64x64x32 cells of the uniform workload); 3-pass kernel: 8.99
 // against 9.00 (64x64x16 cells), 17.88 against 18.03 (shock, 128x32x16), 12.93 against 13.21
-// (bfloat16, 64x64x16).
+// (bfloat16, 64x64x16).  The row-segment kernel keeps form 0; form 1 was not measured there.
 template <bool kLimiter, int kForm = 0>
 struct Walk2 {
     float2 a1, a2, l1, l2, h0, o3;
@@ -385,7 +386,8 @@ struct StepCounters {
     unsigned long long work_next;  // persistent-kernel work counter (fused form)
     unsigned long long pass_next[3];  // work counters of the three passes (3-pass form)
     int error;                     // bit 2: staging wait ran out; bit 3: capacity overflow
-    int done;                      // 1 once every kernel of the step has run
+    int done;                      // set by the step's last kernel as it starts; a 1 that the host
+                                   // reads behind it in the stream means a complete step
     long long needed;              // slots the step's union needed (capacity checks)
 };
 

@@ -696,7 +696,7 @@ vl_status set_blocks(Grid* g, int64_t M, const int64_t* off_in, const uint16_t* 
     Scratch sc(g);
     const int64_t* off = off_in;
     const uint16_t* ids = ids_in;
-    // host values: read in place by the scatter kernel when the buffer is page-locked,
+    // host values: read in place by the kernel of lists.cu when the buffer is page-locked,
     // else streamed through device staging buffers below
     const float* mapped = (!on_device && M > 0) ? static_cast<const float*>(mapped_host(vals_in)) : nullptr;
     const float* vals = on_device ? vals_in : mapped;

@@ -461,189 +461,190 @@ __global__ void __launch_bounds__(kThreads4, 2) k_pass4(PassArgs P)
         }
         int k = k0;
         do {
-        if (!s_any[k] && !s_any[k ^ 1]) continue;  // warp-uniform
+            if (!s_any[k] && !s_any[k ^ 1]) continue;  // warp-uniform
 
-        const bool uni = __all_sync(0xffffffffu, up) || __all_sync(0xffffffffu, !up);
+            const bool uni = __all_sync(0xffffffffu, up) || __all_sync(0xffffffffu, !up);
 
-        const int64_t cin = (int64_t)P.in.base[b] * 4 + (int64_t)q * P.in.cnt[b];    // chunk of rank 0
-        const int64_t cout = (int64_t)P.out.base[b] * 4 + (int64_t)q * P.out.cnt[b];
-        const T* src = static_cast<const T*>(P.in.pool) + cin * kChunk + 4 * vy;
-        T* dst = static_cast<T*>(P.out.pool) + cout * kChunk + 4 * vy;
-        const int* rin = s_rin + k * pitch;
-        const int* rout = s_rout + k * pitch;
-        auto cell_at = [&](int m) { return up ? m : nd - 1 - m; };
-        auto load = [&](int m, float (&o)[4]) {
-            const int r = rin[cell_at(m)];
-            if (r >= 0) {
-                load4<kCodec>(src + (int64_t)r * kChunk, kCodec ? P.in.scale[cin + r] : 1.0f, o);
-            } else {
-                o[0] = o[1] = o[2] = o[3] = 0.0f;
-            }
-        };
-        float t0[4], t1[4];  // originals of walking positions 0 and 1 (the wrapped tail)
-        load(0, t0);
-        load(1 % nd, t1);
-
-        Walk2<kLim, 1> s[2];  // cells (0, 1) and (2, 3) of the row, packed
-        s[0].reset();
-        s[1].reset();
-        float msum = 0.0f;
-        const float thr = P.thr;
-        // every lane calls it for the same position; the 4 lanes of a chunk (one vx row each)
-        // are consecutive, and in place they have all read the chunk at position m - 2 before
-        // the shuffles of that position's call, so its scale may be replaced
-        auto push_emit = [&](int m, const float (&a)[4]) {
-            float res[4];
-            const float2 r01 = s[0].push(make_float2(a[0], a[1]), kp[0]);
-            const float2 r23 = s[1].push(make_float2(a[2], a[3]), kp[1]);
-            res[0] = r01.x;
-            res[1] = r01.y;
-            res[2] = r23.x;
-            res[3] = r23.y;
-            if (m < 2) return;
-            const int c = cell_at(m - 2);
-            const int r = rout[c];
-            T code[4];
-            if constexpr (kCodec != 0) {
-                const float mx = fmaxf(fmaxf(fabsf(res[0]), fabsf(res[1])), fmaxf(fabsf(res[2]), fabsf(res[3])));
-                const ChunkScale cs = chunk_scale(group_max<4>(mx));
-    #pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    code[i] = C::enc(res[i], cs.inv);
-                    if constexpr (kLast) res[i] = C::dec(code[i], cs.s);  // the value the state now holds
+            const int64_t cin = (int64_t)P.in.base[b] * 4 + (int64_t)q * P.in.cnt[b];    // chunk of rank 0
+            const int64_t cout = (int64_t)P.out.base[b] * 4 + (int64_t)q * P.out.cnt[b];
+            const T* src = static_cast<const T*>(P.in.pool) + cin * kChunk + 4 * vy;
+            T* dst = static_cast<T*>(P.out.pool) + cout * kChunk + 4 * vy;
+            const int* rin = s_rin + k * pitch;
+            const int* rout = s_rout + k * pitch;
+            auto cell_at = [&](int m) { return up ? m : nd - 1 - m; };
+            auto load = [&](int m, float (&o)[4]) {
+                const int r = rin[cell_at(m)];
+                if (r >= 0) {
+                    load4<kCodec>(src + (int64_t)r * kChunk, kCodec ? P.in.scale[cin + r] : 1.0f, o);
+                } else {
+                    o[0] = o[1] = o[2] = o[3] = 0.0f;
                 }
-                if (r >= 0 && vy == 0) P.out.scale[cout + r] = cs.s;
-            } else {
-    #pragma unroll
-                for (int i = 0; i < 4; i++) code[i] = res[i];
-            }
-            if (r >= 0) store4<kCodec>(dst + (int64_t)r * kChunk, code);
-            if constexpr (kLast) {
-                const bool keep = r >= 0 && (res[0] >= thr || res[1] >= thr || res[2] >= thr || res[3] >= thr);
-                uint8_t* kq = P.keepq + ((int64_t)P.out.base[b] + r) * 4 + q;
-                if (uni) {
-                    const unsigned bal = __ballot_sync(0xffffffffu, keep);
-                    const unsigned nib = (bal >> ((threadIdx.x & 31) & ~3u)) & 0xfu;  // the chunk's 4 rows
-                    if (nib && vy == 0) *kq = 1;
-                } else if (keep) {
-                    *kq = 1;
-                }
-                if (r >= 0) msum += (res[0] + res[1]) + (res[2] + res[3]);
-            }
-        };
-        // list mode: a batch of positions m .. m+7 is skipped when positions m-10 .. m+7 hold
-        // no output slot in any lane's pencil: the walk has then pushed at least 8 zeros, so
-        // its state is zero and stays so, and every position the batch would emit has no slot
-        auto idle = [&](int m) -> bool {
-            bool quiet = false;
-            if (m >= 10) {
-                const int c0 = up ? m - 10 : nd - m - 8;  // cells c0 .. c0+17
-                const uint32_t* mk = s_slot + k * nw;
-                const int w0 = c0 >> 5;
-                uint64_t v = mk[w0];
-                if (w0 + 1 < nw) v |= (uint64_t)mk[w0 + 1] << 32;
-                quiet = ((v >> (c0 & 31)) & 0x3ffffull) == 0ull;
-            }
-            return __all_sync(0xffffffffu, quiet);
-        };
-        int m = -3;
-        if constexpr (kList) {
-            for (; m < 0; m++) {
-                float a[4];
-                load(wrapi(m, nd), a);
-                s[0].push(make_float2(a[0], a[1]), kp[0]);
-                s[1].push(make_float2(a[2], a[3]), kp[1]);
-            }
-        } else {
-            // the three loads in flight together (uniform 64x64x16 cells 10.36 -> 10.22 ms per step;
-            // in list mode the registers cost more than the latency: shock 21.08 -> 21.18)
-            float a[3][4];
+            };
+            float t0[4], t1[4];  // originals of walking positions 0 and 1 (the wrapped tail)
+            load(0, t0);
+            load(1 % nd, t1);
+
+            Walk2<kLim, 1> s[2];  // cells (0, 1) and (2, 3) of the row, packed
+            s[0].reset();
+            s[1].reset();
+            float msum = 0.0f;
+            const float thr = P.thr;
+            // every lane calls it for the same position; the 4 lanes of a chunk (one vx row each)
+            // are consecutive, and in place they have all read the chunk at position m - 2 before
+            // the shuffles of that position's call, so its scale may be replaced
+            auto push_emit = [&](int m, const float (&a)[4]) {
+                float res[4];
+                const float2 r01 = s[0].push(make_float2(a[0], a[1]), kp[0]);
+                const float2 r23 = s[1].push(make_float2(a[2], a[3]), kp[1]);
+                res[0] = r01.x;
+                res[1] = r01.y;
+                res[2] = r23.x;
+                res[3] = r23.y;
+                if (m < 2) return;
+                const int c = cell_at(m - 2);
+                const int r = rout[c];
+                T code[4];
+                if constexpr (kCodec != 0) {
+                    const float mx = fmaxf(fmaxf(fabsf(res[0]), fabsf(res[1])), fmaxf(fabsf(res[2]), fabsf(res[3])));
+                    const ChunkScale cs = chunk_scale(group_max<4>(mx));
 #pragma unroll
-            for (int u = 0; u < 3; u++) load(wrapi(u - 3, nd), a[u]);
-#pragma unroll
-            for (int u = 0; u < 3; u++) {
-                s[0].push(make_float2(a[u][0], a[u][1]), kp[0]);
-                s[1].push(make_float2(a[u][2], a[u][3]), kp[1]);
-            }
-            m = 0;
-        }
-        if constexpr (kCodec == 0) {
-            for (; m + kBatch4 <= nd; m += kBatch4) {
-                if (kList && idle(m)) continue;
-                float a[kBatch4][4];
-    #pragma unroll
-                for (int u = 0; u < kBatch4; u++) load(m + u, a[u]);
-                // L2 prefetch of the next batch (one lane per chunk row): DRAM keeps working
-                // while this batch's arithmetic runs, and the next loads hit L2.  It takes no
-                // registers; a distance of one batch measured best (0.88 of the copy
-                // bandwidth against 0.76 without, 0.85 at two batches).
-                if (vy == 0) {
-    #pragma unroll
-                    for (int u = 0; u < kBatch4; u++) {
-                        const int pm = m + kBatch4 + u;
-                        if (pm < nd) {
-                            const int r = rin[cell_at(pm)];
-                            if (r >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (int64_t)r * kChunk));
-                        }
+                    for (int i = 0; i < 4; i++) {
+                        code[i] = C::enc(res[i], cs.inv);
+                        if constexpr (kLast) res[i] = C::dec(code[i], cs.s);  // the value the state now holds
                     }
+                    if (r >= 0 && vy == 0) P.out.scale[cout + r] = cs.s;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; i++) code[i] = res[i];
                 }
-    #pragma unroll
-                for (int u = 0; u < kBatch4; u++) push_emit(m + u, a[u]);
+                if (r >= 0) store4<kCodec>(dst + (int64_t)r * kChunk, code);
                 if constexpr (kLast) {
-                    mass += (double)msum;
-                    msum = 0.0f;
+                    const bool keep = r >= 0 && (res[0] >= thr || res[1] >= thr || res[2] >= thr || res[3] >= thr);
+                    uint8_t* kq = P.keepq + ((int64_t)P.out.base[b] + r) * 4 + q;
+                    if (uni) {
+                        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                        const unsigned nib = (bal >> ((threadIdx.x & 31) & ~3u)) & 0xfu;  // the chunk's 4 rows
+                        if (nib && vy == 0) *kq = 1;
+                    } else if (keep) {
+                        *kq = 1;
+                    }
+                    if (r >= 0) msum += (res[0] + res[1]) + (res[2] + res[3]);
                 }
+            };
+            // list mode: a batch of positions m .. m+7 is skipped when positions m-10 .. m+7 hold
+            // no output slot in any lane's pencil: the walk has then pushed at least 8 zeros, so
+            // its state is zero and stays so, and every position the batch would emit has no slot
+            auto idle = [&](int m) -> bool {
+                bool quiet = false;
+                if (m >= 10) {
+                    const int c0 = up ? m - 10 : nd - m - 8;  // cells c0 .. c0+17
+                    const uint32_t* mk = s_slot + k * nw;
+                    const int w0 = c0 >> 5;
+                    uint64_t v = mk[w0];
+                    if (w0 + 1 < nw) v |= (uint64_t)mk[w0 + 1] << 32;
+                    quiet = ((v >> (c0 & 31)) & 0x3ffffull) == 0ull;
+                }
+                return __all_sync(0xffffffffu, quiet);
+            };
+            int m = -3;
+            if constexpr (kList) {
+                for (; m < 0; m++) {
+                    float a[4];
+                    load(wrapi(m, nd), a);
+                    s[0].push(make_float2(a[0], a[1]), kp[0]);
+                    s[1].push(make_float2(a[2], a[3]), kp[1]);
+                }
+            } else {
+                // the three loads in flight together (uniform 64x64x16 cells 10.36 -> 10.22 ms per step;
+                // in list mode the registers cost more than the latency: shock 21.08 -> 21.18)
+                float a[3][4];
+#pragma unroll
+                for (int u = 0; u < 3; u++) load(wrapi(u - 3, nd), a[u]);
+#pragma unroll
+                for (int u = 0; u < 3; u++) {
+                    s[0].push(make_float2(a[u][0], a[u][1]), kp[0]);
+                    s[1].push(make_float2(a[u][2], a[u][3]), kp[1]);
+                }
+                m = 0;
             }
-        } else {
-            // 16-bit storage: the batch is held as raw codes and scales (3 registers per
-            // position instead of 4) and decoded as it is pushed; the next batch's code
-            // sectors and scales are prefetched into L2 like the FP32 rows (50.4 against 64.3
-            // ms per bfloat16 step without; batches of 12 positions measured 52.6 ms)
-            for (; m + kBatch4 <= nd; m += kBatch4) {
-                if (kList && idle(m)) continue;
-                uint2 raw[kBatch4];
-                float sc[kBatch4];
-    #pragma unroll
-                for (int u = 0; u < kBatch4; u++) {
-                    const int r = rin[cell_at(m + u)];
-                    raw[u] = r >= 0 ? *reinterpret_cast<const uint2*>(src + (int64_t)r * kChunk) : make_uint2(0u, 0u);
-                    sc[u] = r >= 0 ? P.in.scale[cin + r] : 0.0f;
-                }
-                if (vy == 0) {
-    #pragma unroll
-                    for (int u = 0; u < kBatch4; u++) {
-                        const int pm = m + kBatch4 + u;
-                        if (pm < nd) {
-                            const int r = rin[cell_at(pm)];
-                            if (r >= 0) {
-                                asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (int64_t)r * kChunk));
-                                asm volatile("prefetch.global.L2 [%0];" ::"l"(P.in.scale + cin + r));
+            if constexpr (kCodec == 0) {
+                for (; m + kBatch4 <= nd; m += kBatch4) {
+                    if (kList && idle(m)) continue;
+                    float a[kBatch4][4];
+#pragma unroll
+                    for (int u = 0; u < kBatch4; u++) load(m + u, a[u]);
+                    // L2 prefetch of the next batch (one lane per chunk row): DRAM keeps working
+                    // while this batch's arithmetic runs, and the next loads hit L2.  It takes no
+                    // registers; a distance of one batch measured best (0.88 of the copy
+                    // bandwidth against 0.76 without, 0.85 at two batches).
+                    if (vy == 0) {
+#pragma unroll
+                        for (int u = 0; u < kBatch4; u++) {
+                            const int pm = m + kBatch4 + u;
+                            if (pm < nd) {
+                                const int r = rin[cell_at(pm)];
+                                if (r >= 0)
+                                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (int64_t)r * kChunk));
                             }
                         }
                     }
+#pragma unroll
+                    for (int u = 0; u < kBatch4; u++) push_emit(m + u, a[u]);
+                    if constexpr (kLast) {
+                        mass += (double)msum;
+                        msum = 0.0f;
+                    }
                 }
-    #pragma unroll
-                for (int u = 0; u < kBatch4; u++) {
-                    float a[4];
-                    const T* h = reinterpret_cast<const T*>(&raw[u]);
-    #pragma unroll
-                    for (int i = 0; i < 4; i++) a[i] = C::dec(h[i], sc[u]);
-                    push_emit(m + u, a);
-                }
-                if constexpr (kLast) {
-                    mass += (double)msum;
-                    msum = 0.0f;
+            } else {
+                // 16-bit storage: the batch is held as raw codes and scales (3 registers per
+                // position instead of 4) and decoded as it is pushed; the next batch's code
+                // sectors and scales are prefetched into L2 like the FP32 rows (50.4 against 64.3
+                // ms per bfloat16 step without; batches of 12 positions measured 52.6 ms)
+                for (; m + kBatch4 <= nd; m += kBatch4) {
+                    if (kList && idle(m)) continue;
+                    uint2 raw[kBatch4];
+                    float sc[kBatch4];
+#pragma unroll
+                    for (int u = 0; u < kBatch4; u++) {
+                        const int r = rin[cell_at(m + u)];
+                        raw[u] = r >= 0 ? *reinterpret_cast<const uint2*>(src + (int64_t)r * kChunk) : make_uint2(0u, 0u);
+                        sc[u] = r >= 0 ? P.in.scale[cin + r] : 0.0f;
+                    }
+                    if (vy == 0) {
+#pragma unroll
+                        for (int u = 0; u < kBatch4; u++) {
+                            const int pm = m + kBatch4 + u;
+                            if (pm < nd) {
+                                const int r = rin[cell_at(pm)];
+                                if (r >= 0) {
+                                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (int64_t)r * kChunk));
+                                    asm volatile("prefetch.global.L2 [%0];" ::"l"(P.in.scale + cin + r));
+                                }
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kBatch4; u++) {
+                        float a[4];
+                        const T* h = reinterpret_cast<const T*>(&raw[u]);
+#pragma unroll
+                        for (int i = 0; i < 4; i++) a[i] = C::dec(h[i], sc[u]);
+                        push_emit(m + u, a);
+                    }
+                    if constexpr (kLast) {
+                        mass += (double)msum;
+                        msum = 0.0f;
+                    }
                 }
             }
-        }
-        for (; m < nd; m++) {
-            float a[4];
-            load(m, a);
-            push_emit(m, a);
-        }
-        push_emit(m, t0);
-        push_emit(m + 1, t1);
-        if constexpr (kLast) mass += (double)msum;
+            for (; m < nd; m++) {
+                float a[4];
+                load(m, a);
+                push_emit(m, a);
+            }
+            push_emit(m, t0);
+            push_emit(m + 1, t1);
+            if constexpr (kLast) mass += (double)msum;
         } while (kMany && (k += kPen4) < npi);
     }
     if constexpr (kLast) {
@@ -720,7 +721,9 @@ vl_status run_3pass(Grid* g, const StepArgs& a)
         // 64x64x16 8.87, 9.00, 9.00.  With one group, before the sweep constants came from a
         // table, 23.4 and 11.2 against 21.2 and 10.3.
         int mult = 1;
-        while (vec && g->codec == 0 && 2 * mult * G.n[d] <= kItemCells && npen * G.nb / (kPen4 * 2 * mult) >= 16 * (int64_t)nsm) mult *= 2;
+        while (vec && g->codec == 0 && 2 * mult * G.n[d] <= kItemCells &&
+               npen * G.nb / (kPen4 * 2 * mult) >= 16 * (int64_t)nsm)
+            mult *= 2;
         P.lg_pen = 4;
         for (int i = mult; i > 1; i >>= 1) P.lg_pen++;
         const int per_cta = vec ? kPen4 * mult : kPencils;
