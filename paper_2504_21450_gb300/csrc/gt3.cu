@@ -374,6 +374,9 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
     const float* ipool = static_cast<const float*>(P.in.pool);
     auto plane_of = [&](int s) { return it.up2 ? s - kHalo : n2 + 2 - s; };
     auto out_of = [&](int s) { return it.up2 ? s - kFirst : n2 + 4 - s; };
+    // this thread's half of a tile row whose output slots it writes below
+    const int oj = sw / (2 * kT), orr = (sw >> 1) - oj * kT;
+    const bool slots = !it.dense_out && sw < nj * 2 * kT && kNB * k + oj >= kFirst;
     if constexpr (kCodec != 0) {
         using T = typename Codec<kCodec>::T;
         const T* cpool = static_cast<const T*>(P.in.pool) + it.ibase;  // codes of rank 0
@@ -542,9 +545,8 @@ __device__ __forceinline__ void stage_batch(const Gt3Args& P, Gt3Smem& S, const 
     // output slots of the tile cells of a sparse next layout, two threads per tile row.  (Read
     // before the copies are issued, with the thread's arrival after the stores, the bitmap
     // words cost registers on every state: 8.73 against 8.71 ms a sweep in bfloat16, 64x64x16
-    // cells of the uniform workload, 15.99 against 15.94 on 128x32x16 of the shock.)
-    const int oj = sw / (2 * kT), orr = (sw >> 1) - oj * kT;
-    if (!it.dense_out && sw < nj * 2 * kT && kNB * k + oj >= kFirst) {
+    // cells of the uniform workload, 15.99 against 15.97 on 128x32x16 of the shock.)
+    if (slots) {
         uint64_t uw = 0ull;
         uint32_t ow = 0u;
         if (orr < it.er) {
